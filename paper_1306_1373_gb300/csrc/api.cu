@@ -75,17 +75,27 @@ static const uint16_t kChromaBase[64] = {
     99, 99, 99, 99, 99, 99, 99, 99,  99, 99, 99, 99, 99, 99, 99, 99};
 
 // Per-output gain of one pass relative to sqrt(8) * orthonormal DCT:
-// [1, K, K/sqrt2, K/sqrt2, 1, K/sqrt2, K/sqrt2, K], K = prod sqrt(1 + 4^-i).
-static void pass_gains(double g[8]) {
-    double k = 1.0;
-    for (int i = 1; i <= kN; ++i) k *= std::sqrt(1.0 + std::ldexp(1.0, -2 * i));
-    const double kr = k / std::sqrt(2.0);
-    const double v[8] = {1.0, k, kr, kr, 1.0, kr, kr, k};
-    for (int i = 0; i < 8; ++i) g[i] = v[i];
-}
+// [1, K, K/sqrt2, K/sqrt2, 1, K/sqrt2, K/sqrt2, K], K = prod sqrt(1 + 4^-i);
+// gg[u * 8 + v] = g_u g_v, and W = rint(2^R / (g_u g_v)), which no quality
+// changes.
+struct Gains {
+    double gg[64];
+    int32_t W[64];
+    Gains() {
+        double k = 1.0;
+        for (int i = 1; i <= kN; ++i) k *= std::sqrt(1.0 + std::ldexp(1.0, -2 * i));
+        const double kr = k / std::sqrt(2.0);
+        const double g[8] = {1.0, k, kr, kr, 1.0, kr, kr, k};
+        for (int u = 0; u < 8; ++u)
+            for (int v = 0; v < 8; ++v) {
+                gg[u * 8 + v] = g[u] * g[v];
+                W[u * 8 + v] = (int32_t)std::nearbyint(std::ldexp(1.0, kR) / gg[u * 8 + v]);
+            }
+    }
+};
 
-dct_status build_tables(int quality, const uint16_t* qtab, int qtab_entries, int chroma, QuantSet& out) {
-    int q[64];
+// Quantiser steps 1..255 of one plane.
+static dct_status quant_steps(int quality, const uint16_t* qtab, int qtab_entries, int chroma, int (&q)[64]) {
     if (quality < 0 || quality > 100) return fail(DCT_ERR_INVALID_ARG, "quality must be 0..100");
     if (quality == 0) {
         if (!qtab) return fail(DCT_ERR_INVALID_ARG, "quality 0 needs qtab_host");
@@ -105,26 +115,58 @@ dct_status build_tables(int quality, const uint16_t* qtab, int qtab_entries, int
             q[i] = v < 1 ? 1 : (v > 255 ? 255 : v);
         }
     }
-    double g[8];
-    pass_gains(g);
-    for (int u = 0; u < 8; ++u) {
-        for (int v = 0; v < 8; ++v) {
-            const int i = u * 8 + v;
-            const double gg = g[u] * g[v];
-            // M = rint(2^32 / (8 * 2^P * gg * Q)); the power of two is exact
-            const double den = gg * (double)q[i];
-            const double m = std::nearbyint(std::ldexp(1.0, kQuantShift - 3 - kP) / den);
-            const double w = std::nearbyint(std::ldexp(1.0, kR) / gg);
-            out.Q[i] = q[i];
-            out.M[i] = (uint32_t)m;
-            out.W[i] = (int32_t)w;
-            out.QW[i] = q[i] * (int32_t)w;
-            // the kernels quantise the non-tie entries without the sign term,
-            // which is exact only while M has at most 11 trailing zero bits
-            // (tie_entry); every Q in 1..255 satisfies this
-            if (!tie_entry(u, v) && (out.M[i] & kTieFreeBits) == 0)
-                return fail(DCT_ERR_UNSUPPORTED, "quantiser multiplier outside the tie-free range");
+    return DCT_OK;
+}
+
+static const Gains& gains() {
+    static const Gains g;
+    return g;
+}
+
+// Quantiser multiplier M = rint(2^32 / (8 * 2^P * gg * Q)) of entry i (the
+// power of two is exact).  The integer quantiser leaves out the sign term off
+// the tie entries, which is exact only while M has at most 11 trailing zero
+// bits (tie_entry); every Q in 1..255 satisfies this.
+static bool multiplier(const Gains& g, int i, int q, uint32_t& m) {
+    m = (uint32_t)std::nearbyint((double)(1ull << (kQuantShift - 3 - kP)) / (g.gg[i] * (double)q));
+    return tie_entry(i >> 3, i & 7) || (m & kTieFreeBits) != 0;
+}
+static dct_status tie_fail() { return fail(DCT_ERR_UNSUPPORTED, "quantiser multiplier outside the tie-free range"); }
+
+dct_status build_tables(int quality, const uint16_t* qtab, int qtab_entries, int chroma, QuantSet& out) {
+    int q[64];
+    dct_status st = quant_steps(quality, qtab, qtab_entries, chroma, q);
+    if (st != DCT_OK) return st;
+    const Gains& g = gains();
+    bool exact = true;
+    for (int i = 0; i < 64; ++i) {
+        if (!multiplier(g, i, q[i], out.M[i])) return tie_fail();
+        out.Q[i] = q[i];
+        out.W[i] = g.W[i];
+        out.QWi[i] = q[i] * g.W[i];
+        out.QW[i] = (float)out.QWi[i];
+        out.QWc[i] = kMagic * (1.0f - out.QW[i]);
+        exact = quant_multiplier(out.M[i], out.Mf[i]) && exact;
+    }
+    if (!exact) out.Mf[0] = 0.0f;
+    return DCT_OK;
+}
+
+dct_status build_tab_args(int quality, const uint16_t* qtab, int qtab_entries, bool chroma, TabArgs& out) {
+    const Gains& g = gains();
+    for (int t = 0; t < (chroma ? 2 : 1); ++t) {
+        int q[64];
+        dct_status st = quant_steps(quality, qtab, qtab_entries, t, q);
+        if (st != DCT_OK) return st;
+        for (int i = 0; i < 64; ++i) {
+            if (!multiplier(g, i, q[i], out.M[t][i])) return tie_fail();
+            out.Q[t][i] = (uint8_t)q[i];
         }
+    }
+    for (int i = 0; i < 64; ++i) out.W[i] = (uint16_t)g.W[i];
+    if (!chroma) {
+        memcpy(out.M[1], out.M[0], sizeof out.M[0]);
+        memcpy(out.Q[1], out.Q[0], sizeof out.Q[0]);
     }
     return DCT_OK;
 }
@@ -280,10 +322,8 @@ static dct_status prepare_planes(dct_plan_t plan, const dct_plane* planes, int n
     if (!planes) return fail(DCT_ERR_INVALID_ARG, "null planes");
     if (nplanes < 1 || nplanes > kMaxPlanes) return fail(DCT_ERR_INVALID_ARG, "nplanes must be 1..4");
     memset(&a, 0, sizeof a);
-    dct_status st = build_tables(quality, qtab, qtab_entries, 0, a.tabs[0]);
-    if (st != DCT_OK) return st;
     const bool yuv = plan->desc.layout == DCT_LAYOUT_YUV420;
-    st = build_tables(quality, qtab, qtab_entries, yuv ? 1 : 0, a.tabs[1]);
+    dct_status st = build_tab_args(quality, qtab, qtab_entries, yuv, a.tabs);
     if (st != DCT_OK) return st;
     int cursor = 0;
     for (int i = 0; i < nplanes; ++i) {

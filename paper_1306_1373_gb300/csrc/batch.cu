@@ -153,14 +153,14 @@ __global__ void __launch_bounds__(256, DCTGB_MINB) k_batch(const __grid_constant
 template <unsigned MODE, int CHUNK>
 __global__ void __launch_bounds__(256, DCTGB_PAIR_MINB) k_batch_pair(const __grid_constant__ BatchArgs args) {
     extern __shared__ __align__(16) uint8_t smem[];
-    constexpr int kWarpBytes = pair_warp_smem_bytes();
+    constexpr int kWarpBytes = pair_warp_smem_bytes(MODE);
+    constexpr int kTabBytes = pair_tab_bytes(MODE);
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int warps_per_cta = blockDim.x >> 5;
     uint8_t* base = smem + (size_t)warp * kWarpBytes;
-    QuantSet* T = reinterpret_cast<QuantSet*>(base);
-    PlaneArg& P = *reinterpret_cast<PlaneArg*>(base + sizeof(QuantSet));
-    uint8_t* xb = base + sizeof(QuantSet) + kDescBytes;
+    PlaneArg& P = *reinterpret_cast<PlaneArg*>(base + kTabBytes);
+    uint8_t* xb = base + kTabBytes + kDescBytes;
 
     const bool claim = args.next_tile != nullptr;
     int tile = 0, limit = 0;
@@ -195,12 +195,13 @@ __global__ void __launch_bounds__(256, DCTGB_PAIR_MINB) k_batch_pair(const __gri
             item_sse = gi->sse;
             if (lane < (int)(sizeof(PlaneArg) / 4))
                 reinterpret_cast<uint32_t*>(&P)[lane] = __ldg(reinterpret_cast<const uint32_t*>(gi) + lane);
-            const uint4* s = reinterpret_cast<const uint4*>(args.tabs + __ldg(&gi->table));
-            uint4* d = reinterpret_cast<uint4*>(T);
-            for (int i = lane; i < (int)(sizeof(QuantSet) / 16); i += 32) d[i] = __ldg(s + i);
+            const uint4* s = reinterpret_cast<const uint4*>(
+                reinterpret_cast<const uint8_t*>(args.tabs + __ldg(&gi->table)) + pair_tab_first(MODE));
+            uint4* d = reinterpret_cast<uint4*>(base);
+            for (int i = lane; i < kTabBytes / 16; i += 32) d[i] = __ldg(s + i);
             __syncwarp();
         }
-        sse += process_tile_pair<MODE>(P, *T, tile - P.tile_begin, lane, xb);
+        sse += process_tile_pair<MODE>(P, pair_tabs<MODE>(base), tile - P.tile_begin, lane, xb);
     }
     if ((MODE & kSse) && cur >= 0 && lane == 0 && sse) atomicAdd(item_sse, sse);
 }
@@ -228,7 +229,6 @@ using KernelPtr = void (*)(BatchArgs);
 template <int C>
 static KernelPtr pair_kernel_c(unsigned mode) {
     switch (mode) {
-        case kLoadPix | kStoreCoef: return k_batch_pair<kLoadPix | kStoreCoef, C>;
         case kLoadCoef | kInverse | kStoreRecon: return k_batch_pair<kLoadCoef | kInverse | kStoreRecon, C>;
         case kLoadCoef | kInverse | kStoreRecon | kSse: return k_batch_pair<kLoadCoef | kInverse | kStoreRecon | kSse, C>;
         case kLoadCoef | kInverse | kStoreRecon | kOwnCodes:
@@ -259,7 +259,9 @@ static KernelPtr pair_kernel(unsigned mode, bool chunked = false) {
 }
 
 // Two lanes per block when the shape asks for it and the mode has a two-lane
-// kernel; one lane per block otherwise.
+// kernel; one lane per block otherwise (the statistics modes, and the forward
+// pass alone: 66.7 us one lane per block, 72.8 us two, on 8192 x 8192 + 4K
+// 4:2:0).
 static bool use_pair(unsigned mode, const dct_launch_shape& sh) {
     return sh.lanes_per_block == 2 && pair_kernel(mode) != nullptr;
 }
@@ -353,7 +355,7 @@ static dct_status ensure_state(dct_plan_t plan) {
 }
 
 static size_t batch_smem(int threads, unsigned mode, const dct_launch_shape& sh) {
-    return (size_t)(threads / 32) * (use_pair(mode, sh) ? pair_warp_smem_bytes() : warp_smem_bytes(mode));
+    return (size_t)(threads / 32) * (use_pair(mode, sh) ? pair_warp_smem_bytes(mode) : warp_smem_bytes(mode));
 }
 
 static int batch_grid(const dct_plan_s* plan, unsigned mode, const dct_launch_shape& sh, int ntiles) {
@@ -609,12 +611,12 @@ dct_status dct_autotune(dct_plan_t plan, dct_launch_shape* best, float* ms_host,
         cudaGetLastError();
     // candidate shapes: CTA sizes x CTAs per SM (beyond the resident count the
     // grid is simply oversubscribed: more, shorter contiguous tile ranges)
-    // and, where the prepared operation has a two-lane kernel, both lanes
+    // and, where one of the prepared kernels has a two-lane form, both lanes
     // per block
     const int threads_c[] = {64, 128, 256};
     const int per_sm_c[] = {1, 2, 4, 8, 16};
-    bool pair_ok = true;
-    for (int k = 0; k < plan->batch->nkernels; ++k) pair_ok = pair_ok && pair_kernel(plan->batch->modes[k]) != nullptr;
+    bool pair_ok = false;
+    for (int k = 0; k < plan->batch->nkernels; ++k) pair_ok = pair_ok || pair_kernel(plan->batch->modes[k]) != nullptr;
     const int nlanes = pair_ok ? 2 : 1;
     dct_launch_shape best_sh = plan->batch->shape;
     float best_ms = 1e30f;

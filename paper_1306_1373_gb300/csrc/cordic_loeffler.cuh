@@ -23,13 +23,9 @@
 
 namespace dctgb {
 
-// acc + (v >> I) with an arithmetic (floor) shift: a shift and an add, both
-// at the full integer issue rate on this GPU (dct_int_peak kind 0 measures
-// 127 of 128 operations per clock per SM).  A single mad.hi.s32 computes
-// the same value (the high word of v * 2^(32-I)), but it issues at about a
-// quarter of that rate: using it for one half of each micro-rotation
-// (dct_int_peak kind 1) measured 80 operations per clock per SM, and made
-// the fused codec step 29% slower with byte-identical outputs.
+// acc + (v >> I) with an arithmetic (floor) shift: one instruction of the
+// integer ALU, acc - (v >> I) two.  (A mad.hi.s32 computes the same value, the
+// high word of v * 2^(32-I), at about a quarter of that rate: dct_int_peak.)
 template <int I>
 __device__ __forceinline__ int add_shr(int acc, int v) {
     return acc + (v >> I);
@@ -77,29 +73,44 @@ __device__ __forceinline__ void cordic_tr_from(int& a, int& b) {
     }
 }
 
-// ---- Forward micro-rotations 2..kN in float32 --------------------------
-// Every float32 of magnitude in [2^23, 2^24) is an integer, and a fused
-// multiply-add rounds its exact result once.  Hold a and b as the floats
-// A = alpha + a and B = beta + b, with compile-time biases alpha, beta in
-// that range (either sign) and beta * 2^-i, alpha * 2^-i integers; then
+// Constants added to a pair (a, b).
+struct FltBias {
+    long long a, b;
+};
+
+// ---- Forward graph in float32 --------------------------------------------
+// The forward graph's nodes are integers below 2^20, so they are exact in
+// float32: its additions and floor shifts run on the FMA pipes, which take a
+// float operation in half the time of an integer shift or add (measured: 0.26
+// clocks and SM for an FFMA against 0.51 for a shift-add, a permute or an
+// integer multiply-add).  Two vectors run at once in the packed form
+// (add.f32x2, fma.f32x2): a packed operation holds the FMA pipe for two, so
+// the rate is the same, but the code is half as long.  8192 x 8192 + 4K 4:2:0,
+// coefficients out, one lane per block: 83.0 us with integer additions and
+// float micro-rotations 2..N, 74.8 us with everything in plain float32, 66.7
+// us packed; the fused two-lane kernel 152.7 us plain, 140.4 us packed.
+//
+// Floor shifts.  Every float32 of magnitude in [2^23, 2^24) is an integer,
+// and a fused multiply-add rounds its exact result once.  Hold a and b as the
+// floats A = alpha + a and B = beta + b, with compile-time biases alpha, beta
+// in that range (either sign) and beta * 2^-i, alpha * 2^-i integers; then
 //   fma round-down(B,  2^-i, A) = (alpha + beta 2^-i) + a + floor(b / 2^i)
 //   fma round-up  (A, -2^-i, B) = (beta - alpha 2^-i) + b - floor(a / 2^i)
-// exactly, as long as the results stay in the range: one FFMA per half
-// micro-rotation in place of a shift (integer ALU pipe only) and an add.
-// The biases follow the micro-rotations themselves (without floors), so
-// the schedule below is fixed per rotation block and checked at compile
-// time against the forward graph's node bound.  Step 1 (a 26.6 degree turn
-// of the bias vector) stays in integers: no bias pair survives it inside
-// the range.  The inverse graph's nodes reach 2^30 and keep the integer
-// form throughout.
+// exactly, as long as the results stay in the range: one operation per half
+// micro-rotation.  The biases follow the micro-rotations themselves (without
+// floors), so the schedule below is fixed per rotation block and checked at
+// compile time against the forward graph's node bound.  Step 1 (a 26.6
+// degree turn) would carry every bias pair out of the range, so it starts
+// from unbiased values and brings the biases in:
+//   fma round-down(b,  1/2, alpha) = alpha + floor(b / 2), then + a
+//   fma round-up  (a, -1/2, beta)  = beta - floor(a / 2),  then + b
+// with both sums exact (integers of magnitude below 2^24).  In the row pass
+// a and b are multiples of 2^kP = 16, so steps 1 and 2 round nothing and are
+// one linear map: two plain fused multiply-adds per output, biases included.
 constexpr long long kFwdNodeBound = 1LL << 20;   // |node| of the forward graph
                                                  // at kP = 4 (interval
                                                  // propagation: 719380)
 constexpr bool kFltForward = kN <= 6;             // biases need 2^(2+..+kN) | alpha
-
-struct FltBias {
-    long long a, b;
-};
 
 // Bias pair before micro-rotation i (2 <= i <= kN + 1) of a block with
 // directions MASK that starts step 2 with (a0, b0).
@@ -143,37 +154,59 @@ static_assert(!kFltForward || (flt_schedule_ok(kSigOddUpper, kFltOddUpperA, kFlt
                                flt_schedule_ok(kSigEven, kFltEvenA, kFltEvenB)),
               "float micro-rotation bias schedule leaves the exact-integer range");
 
-// Bit image of the float alpha + v: for alpha + v in [2^23, 2^24) the bits
-// are 0x4A800000 + alpha + v; in (-2^24, -2^23] (sign and magnitude) they
-// are 0xCA800000 - alpha - v.
-template <long long ALPHA>
-__device__ __forceinline__ float flt_enc(int v) {
-    if constexpr (ALPHA > 0)
-        return __int_as_float((int)(0x4A800000u + (unsigned)ALPHA + (unsigned)v));
-    else
-        return __int_as_float((int)(0xCA800000u + (unsigned)(-ALPHA) - (unsigned)v));
+// Two float32 in a 64-bit register pair, and the packed instructions.
+struct f2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ f2 f2_pack(float x, float y) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ f2 f2_splat(float k) { return f2_pack(k, k); }
+__device__ __forceinline__ float2 f2_unpack(f2 a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+    return r;
+}
+__device__ __forceinline__ f2 operator+(f2 a, f2 b) {
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f2 operator-(f2 a, f2 b) {
+    f2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f2 f2_fma_rn(f2 a, float k, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(f2_splat(k).v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ f2 f2_fma_rd(f2 a, float k, f2 c) {
+    f2 r;
+    asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(f2_splat(k).v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ f2 f2_fma_ru(f2 a, float k, f2 c) {
+    f2 r;
+    asm("fma.rp.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(f2_splat(k).v), "l"(c.v));
+    return r;
 }
 
-template <long long ALPHA>
-__device__ __forceinline__ int flt_dec(float f) {
-    const unsigned bits = (unsigned)__float_as_int(f);
-    if constexpr (ALPHA > 0)
-        return (int)(bits - (0x4A800000u + (unsigned)ALPHA));
-    else
-        return (int)(0xCA800000u + (unsigned)(-ALPHA) - bits);
-}
-
+// Micro-rotations I..kN on biased values.
 template <unsigned MASK, int I>
-__device__ __forceinline__ void cordic_fwd_flt_from(float& a, float& b) {
+__device__ __forceinline__ void cordic_fwd_flt_from(f2& a, f2& b) {
     if constexpr (I <= kN) {
         constexpr float sc = 1.0f / float(1 << I);   // exact power of two
-        float na, nb;
+        f2 na, nb;
         if constexpr ((MASK >> I) & 1u) {
-            na = __fmaf_rd(b, sc, a);     // a + floor(b / 2^I)
-            nb = __fmaf_ru(a, -sc, b);    // b - floor(a / 2^I)
+            na = f2_fma_rd(b, sc, a);     // a + floor(b / 2^I)
+            nb = f2_fma_ru(a, -sc, b);    // b - floor(a / 2^I)
         } else {
-            na = __fmaf_ru(b, -sc, a);    // a - floor(b / 2^I)
-            nb = __fmaf_rd(a, sc, b);     // b + floor(a / 2^I)
+            na = f2_fma_ru(b, -sc, a);    // a - floor(b / 2^I)
+            nb = f2_fma_rd(a, sc, b);     // b + floor(a / 2^I)
         }
         a = na;
         b = nb;
@@ -181,42 +214,158 @@ __device__ __forceinline__ void cordic_fwd_flt_from(float& a, float& b) {
     }
 }
 
+// A rotation block on unbiased integers in float32; run() leaves the
+// schedule's final biases (end) on the results.  ROW: the row pass (inputs
+// multiples of 2^kP).
 template <unsigned MASK, long long A0, long long B0>
-__device__ __forceinline__ void cordic_fwd_flt(int& a, int& b) {
-    int a1, b1;
-    if constexpr ((MASK >> 1) & 1u) {
-        a1 = add_shr<1>(a, b);
-        b1 = sub_shr<1>(b, a);
-    } else {
-        a1 = sub_shr<1>(a, b);
-        b1 = add_shr<1>(b, a);
+struct FltRotation {
+    static constexpr FltBias end = flt_bias(MASK, A0, B0, kN + 1);
+    template <bool ROW>
+    static __device__ __forceinline__ void run(f2& a, f2& b) {
+        f2 fa, fb;
+        if constexpr (ROW) {
+            static_assert(kP >= 3 && kN >= 2, "steps 1 and 2 must be exact");
+            constexpr float s1 = (MASK >> 1) & 1u ? 1.0f : -1.0f, s2 = (MASK >> 2) & 1u ? 1.0f : -1.0f;
+            constexpr float c = 1.0f - s1 * s2 / 8.0f, k = s1 / 2.0f + s2 / 4.0f;
+            constexpr FltBias e = flt_bias(MASK, A0, B0, 3);
+            fa = f2_fma_rn(a, c, f2_fma_rn(b, k, f2_splat((float)e.a)));
+            fb = f2_fma_rn(b, c, f2_fma_rn(a, -k, f2_splat((float)e.b)));
+            cordic_fwd_flt_from<MASK, 3>(fa, fb);
+        } else {
+            if constexpr ((MASK >> 1) & 1u) {
+                fa = a + f2_fma_rd(b, 0.5f, f2_splat((float)A0));
+                fb = b + f2_fma_ru(a, -0.5f, f2_splat((float)B0));
+            } else {
+                fa = a + f2_fma_ru(b, -0.5f, f2_splat((float)A0));
+                fb = b + f2_fma_rd(a, 0.5f, f2_splat((float)B0));
+            }
+            cordic_fwd_flt_from<MASK, 2>(fa, fb);
+        }
+        a = fa;
+        b = fb;
     }
-    float fa = flt_enc<A0>(a1), fb = flt_enc<B0>(b1);
-    cordic_fwd_flt_from<MASK, 2>(fa, fb);
-    constexpr FltBias e = flt_bias(MASK, A0, B0, kN + 1);
-    a = flt_dec<e.a>(fa);
-    b = flt_dec<e.b>(fb);
+};
+using RotOddUpper = FltRotation<kSigOddUpper, kFltOddUpperA, kFltOddUpperB>;
+using RotOddLower = FltRotation<kSigOddLower, kFltOddLowerA, kFltOddLowerB>;
+using RotEven = FltRotation<kSigEven, kFltEvenA, kFltEvenB>;
+
+__device__ __forceinline__ void loeffler8_fwd(int (&v)[8]);
+
+// Sample k of a little-endian word as the float 2^19 + (p << kP): at 2^19 the
+// last mantissa bit counts 2^-4, so the byte goes straight into the second
+// mantissa byte (one byte permute).  The level-shifted sample (p - 128) << kP
+// is that less kPixBias; the graph is linear up to the rotations and its
+// differences cancel the bias, so only Y0 has to take it off (eight times).
+static_assert(kP == 4, "the sample encoding places the byte at a unit of 2^kP");
+constexpr float kPixBias = 524288.0f + 2048.0f;
+template <int K>
+__device__ __forceinline__ float pix_float(uint32_t word) {
+    return __int_as_float(__byte_perm(word, 0x49000000u, 0x7404u | (K << 4)));
 }
 
-template <unsigned MASK, long long A0 = 0, long long B0 = 0>
-__device__ __forceinline__ void cordic_fwd(int& a, int& b) {
-    if constexpr (kFltForward && (A0 != 0 || B0 != 0))
-        cordic_fwd_flt<MASK, A0, B0>(a, b);
-    else
-        cordic_fwd_from<MASK, 1>(a, b);
+// Forward 8-point graph between its first stage (s[n] = x[n] + x[7-n], d[n] =
+// x[n] - x[7-n]) and its last additions.
+struct FwdNodes {
+    f2 e0, e1, y2, y6, a4, a5, a6, a7;   // y2 and y6 still biased (RotEven::end)
+};
+template <bool ROW>
+__device__ __forceinline__ FwdNodes fwd_nodes(const f2 (&s)[4], const f2 (&d)[4]) {
+    FwdNodes n;
+    n.e0 = s[0] + s[3];
+    n.e1 = s[1] + s[2];
+    n.y2 = s[0] - s[3];
+    n.y6 = s[2] - s[1];                // quarter turn of (e2, e3): (e3, -e2)
+    RotEven::run<ROW>(n.y2, n.y6);
+    n.a4 = d[3];
+    n.a7 = d[0];
+    RotOddUpper::run<ROW>(n.a4, n.a7);
+    n.a4 = n.a4 + f2_splat((float)-RotOddUpper::end.a);
+    n.a7 = n.a7 + f2_splat((float)-RotOddUpper::end.b);
+    n.a5 = d[2];
+    n.a6 = d[1];
+    RotOddLower::run<ROW>(n.a5, n.a6);
+    n.a5 = n.a5 + f2_splat((float)-RotOddLower::end.a);
+    n.a6 = n.a6 + f2_splat((float)-RotOddLower::end.b);
+    return n;
+}
+// The last additions of one vector: y[k] <- Y_k.
+template <bool ROW>
+__device__ __forceinline__ void fwd_last(float e0, float e1, float y2, float y6, float a4, float a5, float a6, float a7,
+                                         float (&y)[8]) {
+    const float b4 = __fadd_rn(a4, a6), b7 = __fadd_rn(a7, a5), y0 = __fadd_rn(e0, e1);
+    y[0] = ROW ? __fadd_rn(y0, -8.0f * kPixBias) : y0;
+    y[4] = __fsub_rn(e0, e1);
+    y[2] = __fadd_rn(y2, (float)-RotEven::end.a);
+    y[6] = __fadd_rn(y6, (float)-RotEven::end.b);
+    y[1] = __fadd_rn(b7, b4);
+    y[7] = __fsub_rn(b7, b4);
+    y[3] = __fsub_rn(a7, a5);
+    y[5] = __fsub_rn(a4, a6);
+}
+
+// Forward 8-point graph of two vectors in float32 (in place: v[k] <- Y_k).
+// ROW: they come from pix_float; else they hold unbiased integers.  Packed
+// between the first and the last additions: those run unpacked, so that each
+// vector stays in registers of its own (rows for 16-byte stores, columns out
+// of row registers) without moves.
+template <bool ROW>
+__device__ __forceinline__ void fwd_two(float (&v0)[8], float (&v1)[8]) {
+    if constexpr (!kFltForward) {       // CORDIC counts without a bias schedule
+        int w0[8], w1[8];
+        const float bias = ROW ? -kPixBias : 0.0f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            w0[i] = __float2int_rn(__fadd_rn(v0[i], bias));
+            w1[i] = __float2int_rn(__fadd_rn(v1[i], bias));
+        }
+        loeffler8_fwd(w0);
+        loeffler8_fwd(w1);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            v0[i] = __int2float_rn(w0[i]);
+            v1[i] = __int2float_rn(w1[i]);
+        }
+    } else {
+        f2 s[4], d[4];
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            s[n] = f2_pack(__fadd_rn(v0[n], v0[7 - n]), __fadd_rn(v1[n], v1[7 - n]));
+            d[n] = f2_pack(__fsub_rn(v0[n], v0[7 - n]), __fsub_rn(v1[n], v1[7 - n]));
+        }
+        const FwdNodes n = fwd_nodes<ROW>(s, d);
+        const float2 e0 = f2_unpack(n.e0), e1 = f2_unpack(n.e1), y2 = f2_unpack(n.y2), y6 = f2_unpack(n.y6);
+        const float2 a4 = f2_unpack(n.a4), a5 = f2_unpack(n.a5), a6 = f2_unpack(n.a6), a7 = f2_unpack(n.a7);
+        fwd_last<ROW>(e0.x, e1.x, y2.x, y6.x, a4.x, a5.x, a6.x, a7.x, v0);
+        fwd_last<ROW>(e0.y, e1.y, y2.y, y6.y, a4.y, a5.y, a6.y, a7.y, v1);
+    }
+}
+
+// Samples of one row (two little-endian words) for the row pass.
+__device__ __forceinline__ void pix_row(const uint32_t (&w)[2], float (&y)[8]) {
+    y[0] = pix_float<0>(w[0]);
+    y[1] = pix_float<1>(w[0]);
+    y[2] = pix_float<2>(w[0]);
+    y[3] = pix_float<3>(w[0]);
+    y[4] = pix_float<0>(w[1]);
+    y[5] = pix_float<1>(w[1]);
+    y[6] = pix_float<2>(w[1]);
+    y[7] = pix_float<3>(w[1]);
+}
+
+// N vectors, two at a time.
+template <bool ROW, int N>
+__device__ __forceinline__ void fwd_vectors(float (&v)[N][8]) {
+    static_assert(N % 2 == 0, "vectors go in pairs");
+#pragma unroll
+    for (int i = 0; i < N; i += 2) fwd_two<ROW>(v[i], v[i + 1]);
 }
 
 template <unsigned MASK>
-__device__ __forceinline__ void cordic_tr(int& a, int& b) { cordic_tr_from<MASK, 1>(a, b); }
+__device__ __forceinline__ void cordic_fwd(int& a, int& b) { cordic_fwd_from<MASK, 1>(a, b); }
 
-// Forward 8-point graph on v[0..7] (in place: v[k] <- Y_k); FLT selects
-// the float form of micro-rotations 2..kN (same results, bit for bit).
-template <bool FLT>
+// Forward 8-point graph on v[0..7] in integers (in place: v[k] <- Y_k), for
+// CORDIC counts without a float bias schedule (kN > 6).
 __device__ __forceinline__ void loeffler8_fwd(int (&v)[8]) {
-    constexpr bool F = FLT && kFltForward;
-    constexpr long long UA = F ? kFltOddUpperA : 0, UB = F ? kFltOddUpperB : 0;
-    constexpr long long LA = F ? kFltOddLowerA : 0, LB = F ? kFltOddLowerB : 0;
-    constexpr long long EA = F ? kFltEvenA : 0, EB = F ? kFltEvenB : 0;
     const int s0 = v[0] + v[7], d0 = v[0] - v[7];
     const int s1 = v[1] + v[6], d1 = v[1] - v[6];
     const int s2 = v[2] + v[5], d2 = v[2] - v[5];
@@ -224,11 +373,11 @@ __device__ __forceinline__ void loeffler8_fwd(int (&v)[8]) {
     const int e0 = s0 + s3, e3 = s0 - s3;
     const int e1 = s1 + s2, e2 = s1 - s2;
     int a4 = d3, a7 = d0;
-    cordic_fwd<kSigOddUpper, UA, UB>(a4, a7);
+    cordic_fwd<kSigOddUpper>(a4, a7);
     int a5 = d2, a6 = d1;
-    cordic_fwd<kSigOddLower, LA, LB>(a5, a6);
+    cordic_fwd<kSigOddLower>(a5, a6);
     int y2 = e3, y6 = -e2;             // quarter turn of (e2, e3)
-    cordic_fwd<kSigEven, EA, EB>(y2, y6);
+    cordic_fwd<kSigEven>(y2, y6);
     const int b4 = a4 + a6, b6 = a4 - a6;
     const int b7 = a7 + a5, b5 = a7 - a5;
     v[0] = e0 + e1;
@@ -242,19 +391,23 @@ __device__ __forceinline__ void loeffler8_fwd(int (&v)[8]) {
 }
 
 // Transposed (inverse) 8-point graph on v[0..7] (in place: v[n] <- x_n).
-__device__ __forceinline__ void loeffler8_inv(int (&v)[8]) {
-    const int b7 = v[1] + v[7], b4 = v[1] - v[7];
-    const int b5 = v[3], b6 = v[5];
-    int a4 = b4 + b6, a6 = b4 - b6;
-    int a7 = b7 + b5, a5 = b7 - b5;
-    const int e0 = v[0] + v[4], e1 = v[0] - v[4];
-    int p = v[2], q = v[6];
-    cordic_tr<kSigEven>(p, q);
-    const int e2 = -q, e3 = p;         // transposed quarter turn
-    cordic_tr<kSigOddUpper>(a4, a7);   // -> (d3, d0)
-    cordic_tr<kSigOddLower>(a5, a6);   // -> (d2, d1)
-    const int s0 = e0 + e3, s3 = e0 - e3;
-    const int s1 = e1 + e2, s2 = e1 - e2;
+// The inputs carry a constant Z (the bits a float dequantiser leaves, see
+// dequant_bits), which comes off in the three-input additions of the first
+// stage.  dc is added to v[0].
+template <int Z>
+__device__ __forceinline__ void loeffler8_inv(int (&v)[8], int dc) {
+    constexpr unsigned z = (unsigned)Z;
+    const unsigned v0 = v[0], v1 = v[1], v3 = v[3], v4 = v[4], v5 = v[5], v7 = v[7];
+    const unsigned t = v1 + v7, u = v1 - v7;
+    int a7 = (int)(t + v3 - 3u * z), a5 = (int)(t - v3 - z);
+    int a4 = (int)(u + v5 - z), a6 = (int)(u - v5 + z);
+    const int e0 = (int)(v0 + v4 - 2u * z) + dc, e1 = (int)(v0 - v4) + dc;
+    int p = (int)((unsigned)v[2] - z), q = (int)((unsigned)v[6] - z);
+    cordic_tr_from<kSigEven, 1>(p, q);       // e3 = p, e2 = -q (transposed quarter turn)
+    cordic_tr_from<kSigOddUpper, 1>(a4, a7); // -> (d3, d0)
+    cordic_tr_from<kSigOddLower, 1>(a5, a6); // -> (d2, d1)
+    const int s0 = e0 + p, s3 = e0 - p;
+    const int s1 = e1 - q, s2 = e1 + q;
     v[0] = s0 + a7;
     v[7] = s0 - a7;
     v[1] = s1 + a6;
@@ -263,37 +416,6 @@ __device__ __forceinline__ void loeffler8_inv(int (&v)[8]) {
     v[5] = s2 - a5;
     v[3] = s3 + a4;
     v[4] = s3 - a4;
-}
-
-// 2-D forward: rows (points along the column index j), then columns.
-template <bool FLT>
-__device__ __forceinline__ void fwd2d(int (&x)[8][8]) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) loeffler8_fwd<FLT>(x[i]);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        int c[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) c[i] = x[i][j];
-        loeffler8_fwd<FLT>(c);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) x[i][j] = c[i];
-    }
-}
-
-// 2-D inverse: columns first, then rows (the transpose of fwd2d).
-__device__ __forceinline__ void inv2d(int (&x)[8][8]) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        int c[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) c[i] = x[i][j];
-        loeffler8_inv(c);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) x[i][j] = c[i];
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) loeffler8_inv(x[i]);
 }
 
 }  // namespace dctgb

@@ -30,6 +30,10 @@ cudaError_t ws_event_create(cudaEvent_t* e);
 // table (chroma selects K.2); quality 0 takes qtab (64 or 128 entries).
 dct_status build_tables(int quality, const uint16_t* qtab, int qtab_entries, int chroma, QuantSet& out);
 
+// Both table sets of a direct call (without chroma the second set is the
+// first).
+dct_status build_tab_args(int quality, const uint16_t* qtab, int qtab_entries, bool chroma, TabArgs& out);
+
 // Batch and rate-control state live in batch.cu / ratecontrol.cu; the plan
 // only holds pointers to them.
 struct BatchState;

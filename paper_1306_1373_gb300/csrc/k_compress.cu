@@ -7,21 +7,19 @@ namespace dctgb {
 
 template <unsigned MODE>
 static cudaError_t launch_mode(const DirectArgs& a, int num_sms, int threads, cudaStream_t s) {
+    while (threads > 64 && (long long)a.ntiles < (long long)num_sms * (threads / 32)) threads /= 2;
     const size_t smem = codec_smem_bytes(threads);
     cudaError_t e = cudaFuncSetAttribute(k_codec<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int occ = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_codec<MODE>, threads, smem);
     if (e != cudaSuccess) return e;
-    k_codec<MODE><<<persistent_grid(a.ntiles, threads, num_sms, occ), threads, smem, s>>>(a);
+    k_codec<MODE><<<direct_grid(a.ntiles, threads, num_sms, occ), threads, smem, s>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_compress(const DirectArgs& a, bool stats, int num_sms, int threads, cudaStream_t s) {
     if (stats) return launch_mode<kLoadPix | kStoreCoef | kStats>(a, num_sms, threads, s);
-    // one lane per block: its forward pass runs the float micro-rotations
-    // (measured 849 against 803 GPix/s for the two-lane kernel on the
-    // benchmark planes)
     return launch_mode<kLoadPix | kStoreCoef>(a, num_sms, threads, s);
 }
 

@@ -1,6 +1,7 @@
 // Codec kernels: forward path (Sec. 2.5.2 transform + Sec. 3.2 quantiser),
 // inverse path (Sec. 3.2 dequantiser + IDCT) and the SSE of Eq. 24, for
-// uint8 planes, all in integer arithmetic.
+// uint8 planes.  The forward path computes the integers of the flow graph in
+// float32 on the FMA pipes (cordic_loeffler.cuh), the inverse path in int32.
 //
 // Work decomposition: a plane of nbx x nby 8x8 blocks is cut into warp tiles
 // of kTileBlocks consecutive blocks in block-major order (b = by * nbx + bx,
@@ -11,7 +12,7 @@
 // swizzled per-warp shared-memory stage so the global side moves 16 bytes
 // per lane over contiguous 512-byte spans.  The batched kernel prefetches
 // the next tile's pixels / coefficients with cp.async while the current
-// tile computes.  The path is bound by integer issue, not by HBM, so the
+// tile computes.  The path is bound by instruction issue, not by HBM, so the
 // code is arranged to minimise instructions per sample.
 #pragma once
 #include <cstdint>
@@ -32,11 +33,17 @@ constexpr int kStageBytes = kTileBlocks * 128;    // one tile of int16 coefficie
 constexpr int kPixBytes = kTileBlocks * 64;       // one tile of uint8 samples
 
 // Per-plane quantiser / dequantiser tables (natural order u*8+v).
+// The float entries drive the kernels that quantise on the FMA pipes (see
+// quant_code and dequant_bits).
 struct QuantSet {
     uint32_t M[64];   // rint(2^32 / (8 * 2^P * g_u g_v Q))
+    float Mf[64];     // M * 2^-32, with the tie rule of quant_multiplier;
+                      // Mf[0] = 0 when some M does not fit 24 bits
+    float QW[64];     // Q * W
+    float QWc[64];    // kMagic * (1 - Q * W)
+    int32_t QWi[64];  // Q * W
     int32_t Q[64];    // 1..255
     int32_t W[64];    // rint(2^R / (g_u g_v))
-    int32_t QW[64];   // Q * W
 };
 
 struct PlaneArg {
@@ -54,9 +61,17 @@ struct PlaneArg {
 };
 constexpr int kVecSrc = 1, kVecDst = 2, kVecRef = 4;
 
+// What a direct call's kernel needs to build its two table sets (luma,
+// chroma) in shared memory: a launch carries 768 bytes instead of 3.5 KB.
+struct TabArgs {
+    uint32_t M[2][64];
+    uint16_t W[64];
+    uint8_t Q[2][64];
+};
+
 struct DirectArgs {
     PlaneArg p[kMaxPlanes];
-    QuantSet tabs[2];
+    TabArgs tabs;
     int32_t nplanes;
     int32_t ntiles;
 };
@@ -75,27 +90,96 @@ enum : unsigned {
                           // forward kernel of the same graph: the dequantiser clamp never acts
 };
 
-// Forward micro-rotations 2..N in the float form (cordic_loeffler.cuh) for
-// kernels that run the forward transform without the inverse: measured on
-// the benchmark planes, the compress-only pass runs 5-7% faster with it
-// (the FMA pipes take the shift-adds off the integer ALU pipe), while the
-// fused forward + inverse kernel runs 1.7% slower (its instruction count
-// falls only 1.6% and issue drops from 80.6% to 77.8% of cycles), so the
-// fused kernels keep the integer form.
-__host__ __device__ constexpr bool fwd_in_float(unsigned mode) { return (mode & kLoadPix) && !(mode & kInverse); }
-
-// Quantiser entries that can meet an exact rounding tie.  The definition
-// q = sgn(Y) ((|Y| M + 2^31) >> 32) equals the high word of the signed
-// Y M + 2^31 for Y >= 0 always, and for Y < 0 unless |Y| M = 2^31 (mod 2^32),
-// which needs |Y| = 2^(31-k) * odd, k = trailing zero bits of M.  The forward
-// graph keeps |Y| <= 719380 < 2^20 (interval bound), so an entry with k <= 11
-// never ties.  Where u and v are both 0 or 4, g_u g_v = 1 and
-// M = rint(2^25 / Q) is a high power of two for Q = 1, 2, 4, ...: these four
-// entries keep the sign-aware form.  For the other 60, every Q in 1..255
-// gives k <= 11 (build_tables checks each table), so the plain high word is
-// the exact quantiser there: one 64-bit multiply-add per coefficient.
+// ---- quantiser and own-code dequantiser on the FMA pipes ------------------
+//
+// Quantiser.  q = sgn(Y) ((|Y| M + 2^31) >> 32) is Y M / 2^32 rounded to the
+// nearest integer, halves away from zero.  One fused multiply-add with
+// kMagic = 1.5 * 2^23 (where a float32 counts ones) gives kMagic + q: the
+// exact product is rounded once, to the nearest integer, halves to even.
+// The two differ only at exact halves |Y| M = 2^31 (mod 2^32), which need
+// |Y| = 2^(31-k) * odd, k = trailing zero bits of M; the forward graph keeps
+// |Y| <= 719380 < 2^20 (interval bound), so k >= 12.  That happens only where
+// u and v are both 0 or 4 (g_u g_v = 1, M = rint(2^25 / Q) a high power of two
+// for Q = 1, 2, 4, ...); there the multiplier is the next float above
+// M * 2^-32, which lifts the exact halves over the half and moves no other
+// product across one (a test runs every reachable M over every |Y|).
+// M must fit a float's 24 bits: only M > 2^24 (Q = 1, and Q = 2 at the
+// smallest gains; quality 93 and up) may not, and tables with such an entry
+// take the integer form (Mf[0] = 0).  The integer form costs a 64-bit multiply,
+// which issues at 1/8 of the FMA rate (measured: 16 against 128 per clock per
+// SM); this one costs half an issue slot.
+constexpr float kMagic = 12582912.0f;               // 1.5 * 2^23
+constexpr int kMagicBits = 0x4B400000;              // its bits: bits(kMagic + q) = kMagicBits + q
 __host__ __device__ constexpr bool tie_entry(int u, int v) { return (u & 3) == 0 && (v & 3) == 0; }
 constexpr uint32_t kTieFreeBits = 0xFFFu;   // (M & kTieFreeBits) != 0  <=>  k <= 11
+
+// The float multiplier of M (above): false when M needs more than 24 bits.
+__host__ __device__ inline bool quant_multiplier(uint32_t m, float& out) {
+    const float f = (float)m;
+    if ((double)f != (double)m) return false;
+    out = f * 2.3283064365386963e-10f;      // 2^-32
+    if ((m & kTieFreeBits) == 0) {          // the next float above
+        union { float f; uint32_t u; } b;
+        b.f = out;
+        b.u += 1u;
+        out = b.f;
+    }
+    return true;
+}
+
+// Coefficient (u, v) to kMagic + q.
+template <bool FLT, int U, int V>
+__device__ __forceinline__ float quant_code(float y, float mf, const uint32_t* M) {
+    if constexpr (FLT) return __fmaf_rn(y, mf, kMagic);
+    // high word of Y M + 2^31, with - [Y < 0] where halves can occur (M < 2^26)
+    const int yi = __float_as_int(__fadd_rn(y, kMagic)) - kMagicBits;
+    long long p = (long long)yi * (long long)(int)M[U * 8 + V] + 0x80000000ll;
+    if (tie_entry(U, V)) p += (long long)(yi >> 31);
+    return __int_as_float((int)(p >> 32) + kMagicBits);
+}
+
+// An own code kMagic + q, dequantised: G = q (Q W) as the integer kMagicBits +
+// G, in one fused multiply-add: (kMagic + q) (Q W) + kMagic (1 - Q W) (QWc, an
+// exact float: 3 (1 - Q W) 2^22 with Q W < 2^20).  The clamp of the definition
+// never acts on this library's own codes: |q Q| <= |X| + Q/2 + 1 < 1200 (the
+// Cordic coefficient |X| is within 14 of an orthonormal DCT value at kN = 6,
+// itself at most 1024; < 1220 at kN = 4), so |G| < 1220 * 3025 < 2^22 and
+// kMagic + G is an exact float32 integer.
+__device__ __forceinline__ int dequant_bits(float t, float qw, float qwc) {
+    return __float_as_int(__fmaf_rn(t, qw, qwc));
+}
+
+// The two table sets of a direct call, from its arguments into shared memory
+// (every thread of the CTA; ends with a barrier).
+__device__ __forceinline__ void build_tabs(const TabArgs& a, QuantSet* tabs) {
+    bool exact = true;
+    for (int i = threadIdx.x; i < 128; i += blockDim.x) {
+        QuantSet& t = tabs[i >> 6];
+        const int k = i & 63;
+        const uint32_t m = a.M[i >> 6][k];
+        const int q = a.Q[i >> 6][k], w = a.W[k];
+        float mf = 0.0f;
+        exact = quant_multiplier(m, mf) && exact;
+        t.M[k] = m;
+        t.Mf[k] = mf;
+        t.QWi[k] = q * w;
+        t.QW[k] = (float)(q * w);
+        t.QWc[k] = kMagic * (1.0f - (float)(q * w));
+        t.Q[k] = q;
+        t.W[k] = w;
+    }
+    // a set with an inexact entry would need its own flag; both fall back
+    // together, which only costs time
+    if (!__syncthreads_and(exact)) {
+        if (threadIdx.x < 2) tabs[threadIdx.x].Mf[0] = 0.0f;
+        __syncthreads();
+    }
+}
+
+// int16 pair of two codes kMagic + q: their low halves.
+__device__ __forceinline__ uint32_t pack_codes(float t0, float t1) {
+    return __byte_perm((uint32_t)__float_as_int(t0), (uint32_t)__float_as_int(t1), 0x5410);
+}
 
 // Clamp to 0..255 in one instruction: max(min(v, 255), 0).
 __device__ __forceinline__ int clamp_u8(int v) { return __vimin_s32_relu(v, 255); }
@@ -281,6 +365,96 @@ __host__ __device__ constexpr int warp_smem_bytes(unsigned mode) {
 // one warp tile
 // --------------------------------------------------------------------------
 
+// Added once to the DC input, which reaches every output through additions
+// only: the descale rounding term 2^(R+2) and the +128 level.
+constexpr int kDcBias = (1 << (kR + 2)) + (128 << (kR + 3));
+
+// Eight outputs of the inverse row pass, descaled and clamped, to two words.
+__device__ __forceinline__ void descale_row(const int (&v)[8], uint32_t (&out)[2]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        uint32_t wd = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) wd |= (uint32_t)clamp_u8(v[4 * h + k] >> (kR + 3)) << (8 * k);
+        out[h] = wd;
+    }
+}
+
+// Columns V and V + 1 of the forward tile: column pass, band statistics,
+// quantiser (code pairs to w), and in the fused modes dequantiser and inverse
+// column pass (to x).
+template <unsigned MODE, bool FLT, int V, int U = 0>
+__device__ __forceinline__ void fwd_quant_rows(const QuantSet& T, const float (&y0)[8], const float (&y1)[8],
+                                               uint32_t (&w)[8][4], int (&c0)[8], int (&c1)[8]) {
+    if constexpr (U < 8) {
+        const float2 mf = *reinterpret_cast<const float2*>(&T.Mf[U * 8 + V]);
+        const float t0 = quant_code<FLT, U, V>(y0[U], mf.x, T.M), t1 = quant_code<FLT, U, V + 1>(y1[U], mf.y, T.M);
+        if (MODE & kStoreCoef) w[U][V / 2] = pack_codes(t0, t1);
+        if (MODE & kInverse) {
+            const float2 qw = *reinterpret_cast<const float2*>(&T.QW[U * 8 + V]);
+            const float2 qc = *reinterpret_cast<const float2*>(&T.QWc[U * 8 + V]);
+            c0[U] = dequant_bits(t0, qw.x, qc.x);
+            c1[U] = dequant_bits(t1, qw.y, qc.y);
+        }
+        fwd_quant_rows<MODE, FLT, V, U + 1>(T, y0, y1, w, c0, c1);
+    }
+}
+template <unsigned MODE, bool FLT, int V>
+__device__ __forceinline__ void fwd_tile_cols(const QuantSet& T, const float (&f)[8][8], bool active, int lane,
+                                              unsigned long long* st, unsigned& ac, uint32_t (&w)[8][4], int (&x)[8][8]) {
+    float y[2][8];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+#pragma unroll
+        for (int r = 0; r < 8; ++r) y[k][r] = f[r][V + k];
+    }
+    fwd_vectors<false>(y);
+    if (MODE & kStats) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const unsigned a = (unsigned)abs(__float2int_rn(y[k][u])) >> kBandShift;
+                const unsigned e = active ? a * a : 0u;
+                if (u | (V + k)) ac += e;
+                const unsigned tot = warp_sum(e);
+                if (lane == 0) st_add<MODE>(&st[kStBand + u * 8 + V + k], tot);
+            }
+        }
+    }
+    if (!(MODE & (kStoreCoef | kInverse))) return;
+    int c0[8], c1[8];
+    fwd_quant_rows<MODE, FLT, V>(T, y[0], y[1], w, c0, c1);
+    if (MODE & kInverse) {
+        loeffler8_inv<kMagicBits>(c0, V == 0 ? kDcBias : 0);
+        loeffler8_inv<kMagicBits>(c1, 0);
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            x[r][V] = c0[r];
+            x[r][V + 1] = c1[r];
+        }
+    }
+}
+
+// All columns, with the quantiser form of the table: one warp-uniform branch
+// per tile (one per coefficient row cost two instructions a sample and cut
+// the column pass into small pieces).
+template <unsigned MODE>
+__device__ __forceinline__ void fwd_columns(const QuantSet& T, const float (&f)[8][8], bool active, int lane,
+                                            unsigned long long* st, unsigned& ac, uint32_t (&w)[8][4], int (&x)[8][8]) {
+    if (!(MODE & (kStoreCoef | kInverse)) || T.Mf[0] != 0.0f) {
+        fwd_tile_cols<MODE, true, 0>(T, f, active, lane, st, ac, w, x);
+        fwd_tile_cols<MODE, true, 2>(T, f, active, lane, st, ac, w, x);
+        fwd_tile_cols<MODE, true, 4>(T, f, active, lane, st, ac, w, x);
+        fwd_tile_cols<MODE, true, 6>(T, f, active, lane, st, ac, w, x);
+    } else {
+        fwd_tile_cols<MODE, false, 0>(T, f, active, lane, st, ac, w, x);
+        fwd_tile_cols<MODE, false, 2>(T, f, active, lane, st, ac, w, x);
+        fwd_tile_cols<MODE, false, 4>(T, f, active, lane, st, ac, w, x);
+        fwd_tile_cols<MODE, false, 6>(T, f, active, lane, st, ac, w, x);
+    }
+}
+
 // Processes warp tile `tile_in_plane` of plane P.
 //  stage      kStageBytes of this warp's shared memory (coefficients)
 //  pixbuf     this tile's prefetched samples (forward) or SSE reference
@@ -354,27 +528,18 @@ __device__ __forceinline__ unsigned process_tile(const PlaneArg& P, const QuantS
             }
         }
 
-        // level shift: x = (p - 128) << P
+        float f[8][8];
 #pragma unroll
-        for (int r = 0; r < 8; ++r)
-#pragma unroll
-            for (int c = 0; c < 8; ++c) x[r][c] = (sample(pix, r, c) - 128) * (1 << kP);
+        for (int r = 0; r < 8; ++r) pix_row(pix[r], f[r]);
+        fwd_vectors<true>(f);
 
-        fwd2d<fwd_in_float(MODE)>(x);
+        // column pass, two columns at a time: statistics, quantiser, codes
+        // and (fused modes) dequantiser and inverse column pass
+        unsigned ac = 0;
+        uint32_t w[8][4];
+        fwd_columns<MODE>(T, f, active, lane, st, ac, w, x);
 
         if (MODE & kStats) {
-            unsigned ac = 0;
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-#pragma unroll
-                for (int v = 0; v < 8; ++v) {
-                    const unsigned a = (unsigned)abs(x[u][v]) >> kBandShift;
-                    const unsigned e = active ? a * a : 0u;
-                    if (u | v) ac += e;
-                    const unsigned tot = warp_sum(e);
-                    if (lane == 0) st_add<MODE>(&st[kStBand + u * 8 + v], tot);
-                }
-            }
             const unsigned thr[4] = {1u << 10, 1u << 14, 1u << 18, 1u << 22};
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -383,43 +548,10 @@ __device__ __forceinline__ unsigned process_tile(const PlaneArg& P, const QuantS
             }
         }
 
-        // Quantiser q = sgn(Y) ((|Y| M + 2^31) >> 32).  Away from the four
-        // tie entries the high word of Y M + 2^31 is exact (tie_entry).  At
-        // the tie entries the fused kernels use the high word of the signed
-        // Y * M + 2^31 - [Y < 0] (for Y < 0, floor((Y M + 2^31 - 1) / 2^32) =
-        // -floor((|Y| M + 2^31) / 2^32), so both signs round half away from
-        // zero exactly as the definition); the forward-only kernels use |Y|,
-        // an unsigned multiply and the sign.
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-#pragma unroll
-            for (int v = 0; v < 8; ++v) {
-                const int y = x[u][v];
-                if (!tie_entry(u, v)) {
-                    const long long p = (long long)y * (long long)(int)T.M[u * 8 + v] + 0x80000000ll;
-                    x[u][v] = (int)(p >> 32);
-                } else if (MODE & kInverse) {
-                    const unsigned c = 0x80000000u ^ (unsigned)(y >> 31);
-                    const long long p = (long long)y * (long long)(int)T.M[u * 8 + v] + (long long)c;
-                    x[u][v] = (int)(p >> 32);
-                } else {
-                    const uint32_t a = (uint32_t)abs(y);
-                    const uint32_t q = (uint32_t)(((unsigned long long)a * T.M[u * 8 + v] + 0x80000000ull) >> 32);
-                    x[u][v] = y < 0 ? -(int)q : (int)q;
-                }
-            }
-        }
-
         if (MODE & kStoreCoef) {
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                uint4 w;
-                w.x = ((uint32_t)x[u][0] & 0xFFFFu) | ((uint32_t)x[u][1] << 16);
-                w.y = ((uint32_t)x[u][2] & 0xFFFFu) | ((uint32_t)x[u][3] << 16);
-                w.z = ((uint32_t)x[u][4] & 0xFFFFu) | ((uint32_t)x[u][5] << 16);
-                w.w = ((uint32_t)x[u][6] & 0xFFFFu) | ((uint32_t)x[u][7] << 16);
-                *reinterpret_cast<uint4*>(stage + stage_off(lane, u)) = w;
-            }
+            for (int u = 0; u < 8; ++u)
+                *reinterpret_cast<uint4*>(stage + stage_off(lane, u)) = make_uint4(w[u][0], w[u][1], w[u][2], w[u][3]);
             __syncwarp();
             uint4* g = reinterpret_cast<uint4*>(P.coef + (size_t)b0 * 64);
 #pragma unroll
@@ -462,42 +594,33 @@ __device__ __forceinline__ unsigned process_tile(const PlaneArg& P, const QuantS
     }
 
     if (MODE & kInverse) {
-        // Dequantiser G = clamp(q Q, -4096, 4096) W.  When q comes from this
-        // library's quantiser (this kernel's, or the forward kernel's of the
-        // same two-pass graph), |q Q| <= |X| + Q/2 + 1 < 1200 (the Cordic
-        // coefficient |X| is within 14 of an orthonormal DCT value, itself at
-        // most 1024), so the clamp never acts and G = q (Q W) exactly.
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
+        // Dequantiser and inverse column pass of stored codes (the fused
+        // modes did both above).  Codes written by the forward kernel of
+        // the same graph need no clamp (dequant_bits): G = q (Q W).
+        if (!(MODE & kLoadPix)) {
 #pragma unroll
             for (int v = 0; v < 8; ++v) {
-                if (MODE & (kLoadPix | kOwnCodes)) {
-                    x[u][v] = x[u][v] * T.QW[u * 8 + v];
-                } else {
-                    int t = x[u][v] * T.Q[u * 8 + v];
-                    t = max(-kDequantClamp, min(kDequantClamp, t));
-                    x[u][v] = t * T.W[u * 8 + v];
+                int c[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    if (MODE & kOwnCodes) {
+                        c[u] = x[u][v] * T.QWi[u * 8 + v];
+                    } else {
+                        const int t = x[u][v] * T.Q[u * 8 + v];
+                        c[u] = max(-kDequantClamp, min(kDequantClamp, t)) * T.W[u * 8 + v];
+                    }
                 }
+                loeffler8_inv<0>(c, v == 0 ? kDcBias : 0);
+#pragma unroll
+                for (int r = 0; r < 8; ++r) x[r][v] = c[r];
             }
         }
-        // The DC input reaches every output through additions only, so the
-        // descale rounding term 2^(R+2) and the +128 level (128 << (R+3))
-        // are added once here instead of at each of the 64 outputs.
-        x[0][0] += (1 << (kR + 2)) + (128 << (kR + 3));
-        inv2d(x);
+        // inverse row pass, descale and clamp, four samples to a word
         uint32_t out[8][2];
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                uint32_t wd = 0;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int v = clamp_u8(x[r][4 * h + k] >> (kR + 3));
-                    wd |= (uint32_t)v << (8 * k);
-                }
-                out[r][h] = wd;
-            }
+            loeffler8_inv<0>(x[r], 0);
+            descale_row(x[r], out[r]);
         }
         if ((MODE & kStoreRecon) && active)
             store_block(P.dst, P.dst_pitch, P.width, P.height, by, bx, (P.flags & kVecDst) != 0, out);
@@ -549,15 +672,13 @@ __global__ void __launch_bounds__(256, DCTGB_MINB) k_codec(const __grid_constant
 
     // tables -> shared memory
     {
-        const uint32_t* s = reinterpret_cast<const uint32_t*>(args.tabs);
-        uint32_t* d = reinterpret_cast<uint32_t*>(tabs);
-        for (int i = threadIdx.x; i < (int)(2 * sizeof(QuantSet) / 4); i += blockDim.x) d[i] = s[i];
         unsigned long long* a = reinterpret_cast<unsigned long long*>(acc);
         for (int i = threadIdx.x; i < (int)(sizeof(CtaAcc) / 8); i += blockDim.x) a[i] = 0ull;
-        __syncthreads();
-        if (MODE & kStats)
+        build_tabs(args.tabs, tabs);
+        if (MODE & kStats) {
             if (threadIdx.x < kMaxPlanes) acc->st[threadIdx.x][kStMin] = ~0ull;
-        __syncthreads();
+            __syncthreads();
+        }
     }
 
     const int lane = threadIdx.x & 31;
@@ -605,16 +726,32 @@ inline size_t codec_smem_bytes(int threads) {
     return 2 * sizeof(QuantSet) + sizeof(CtaAcc) + (size_t)(threads / 32) * kStageBytes;
 }
 
-// Persistent grid: enough CTAs for every tile, at most num_sms * occupancy.
-inline int persistent_grid(int ntiles, int threads, int num_sms, int occ) {
+// Grid of a direct call: enough CTAs for every unit of work (one warp each);
+// beyond the resident count, a persistent grid of c CTAs per SM, each warp
+// taking every (grid size)-th unit.  Every SM then issues c * rounds units
+// per warp position, so c (at least two thirds of the resident count, to keep
+// the latencies hidden) is the one that wastes the least in the last round: a
+// 4K 4:2:0 frame is 40 tiles per SM, 3 rounds of 14 warps instead of 16.
+inline int direct_grid(int units, int threads, int num_sms, int occ) {
     const int warps = threads / 32;
-    const int need = (ntiles + warps - 1) / warps;
-    const int cap = num_sms * (occ > 0 ? occ : 1);
-    return need < 1 ? 1 : (need < cap ? need : cap);
+    if (occ < 1) occ = 1;
+    const long long need = ((long long)units + warps - 1) / warps;
+    if (need <= (long long)num_sms * occ) return need < 1 ? 1 : (int)need;
+    int best = occ;
+    long long best_cost = 0;
+    for (int c = occ; c >= 1 && 3 * c >= 2 * occ; --c) {
+        const long long per_round = (long long)num_sms * c * warps;
+        const long long cost = (((long long)units + per_round - 1) / per_round) * c;
+        if (best_cost == 0 || cost < best_cost) {
+            best_cost = cost;
+            best = c;
+        }
+    }
+    return num_sms * best;
 }
 
 // host launchers (one translation unit per family); kDirectThreads per CTA
-constexpr int kDirectThreads = 256;
+constexpr int kDirectThreads = 128;
 cudaError_t launch_compress(const DirectArgs& a, bool stats, int num_sms, int threads, cudaStream_t s);
 cudaError_t launch_reconstruct(const DirectArgs& a, bool sse, int num_sms, int threads, cudaStream_t s);
 cudaError_t launch_fused(const DirectArgs& a, bool coef, bool recon, int num_sms, int threads, cudaStream_t s);

@@ -1,20 +1,22 @@
-// Codec tile with two lanes per 8x8 block: the fused pass, the forward pass
-// alone and the inverse pass alone.
+// Codec tile with two lanes per 8x8 block: the fused pass and the inverse pass
+// alone.
 //
-// The one-lane-per-block tile (kernels.cuh) keeps all 64 samples of a block
-// in one thread, which makes the row/column transpose free but needs about
-// 128 registers, so only 16 warps fit on an SM; the path is bound by integer
-// issue, and 16 warps leave about a quarter of the issue slots idle on
-// dependency and pipe-throttle stalls.  Here lanes 2k and 2k+1 share block k
-// of a 16-block half tile: lane h owns rows 4h..4h+3 for the row passes and
-// columns 4h..4h+3 for the column passes, 32 values in registers, and the two
-// transposes go through a padded per-warp shared-memory slot (8 stores and 8
-// loads of 16 bytes per lane each, no bank conflicts).  To stay within 64
-// registers with few spills, the samples wait for the SSE in a per-lane
-// shared-memory slot, and the coefficients go straight from registers to
-// global memory (8 bytes per lane and row: the lane pair fills the row's 16
-// bytes).  The arithmetic is the same integer graph in the same order as the
-// one-lane tile, so every output is bit-identical to it.
+// Lanes 2k and 2k+1 share block k of a 16-block half tile: lane h owns rows
+// 4h..4h+3 for the row passes and columns 4h..4h+3 for the column passes, 32
+// values in registers, and the two transposes go through a padded per-warp
+// shared-memory slot (8 stores and 8 loads of 16 bytes per lane each, no bank
+// conflicts).  Against the one-lane tile (kernels.cuh) this halves the code of
+// a tile and the registers: the fused one-lane kernel is 2700 instructions
+// long and waits for instruction fetches (ncu: 1.5 cycles of "no instruction"
+// per issued one, 0.1 here).  What bounds it is issue (66% of cycles, a packed
+// float instruction holding two), with the integer ALU at 60% and the L1 data
+// path at 56%.  At most 80 registers (24 warps per SM): 138.4 us on 8192 x
+// 8192 + 4K 4:2:0 against 142.4 us at 64 registers (32 warps, spills).  The
+// samples wait for the SSE in a per-lane shared-memory slot, and the codes
+// leave through the transpose buffer, free between the two transposes, so that
+// a store moves 512 contiguous bytes (8 bytes per lane straight from registers
+// touched 16 cache lines per store; the forward pass alone took 83.1 us that
+// way, 72.8 us staged).
 //
 // Transpose slot of block k (kXSlot bytes): row r, column quad q (columns
 // 4q..4q+3, four int32) at k*kXSlot + (r>>2)*kXRowHalf + (r&3)*32 + q*16.
@@ -23,10 +25,12 @@
 // it reads its column quad, so each quarter-warp phase hits 8 distinct
 // groups.
 #pragma once
+#include <cstddef>
+
 #include "kernels.cuh"
 
 #ifndef DCTGB_PAIR_MINB
-#define DCTGB_PAIR_MINB 4   // resident CTAs of 256 threads per SM (launch bounds: <= 64 registers)
+#define DCTGB_PAIR_MINB 3   // resident CTAs of 256 threads per SM (launch bounds: <= 80 registers)
 #endif
 
 namespace dctgb {
@@ -37,20 +41,51 @@ constexpr int kXRowHalf = 144;                    // offset of rows 4..7 in a sl
 constexpr int kXBytes = kPairBlocks * kXSlot;     // per warp
 constexpr int kParkBytes = 32 * 32;               // each lane's 32 samples, kept for the SSE
 
-// Shared memory per warp of the two-lane batched kernel: tables, descriptor,
-// transpose buffer, sample slots.
-__host__ __device__ constexpr int pair_warp_smem_bytes() {
-    return (int)sizeof(QuantSet) + kDescBytes + kXBytes + kParkBytes;
+// The part of a QuantSet that a mode reads: [M, Mf, QW, QWc] forward and fused,
+// [QWi] for the inverse of own codes, [Q, W] for the inverse of any codes.
+// Batched warps keep only that part, so that 32 warps' slots fit an SM.
+__host__ __device__ constexpr int pair_tab_first(unsigned mode) {
+    return (mode & kLoadPix) ? (int)offsetof(QuantSet, M)
+                             : (mode & kOwnCodes) ? (int)offsetof(QuantSet, QWi) : (int)offsetof(QuantSet, Q);
+}
+__host__ __device__ constexpr int pair_tab_bytes(unsigned mode) {
+    return (mode & kLoadPix) ? 4 * 256 : (mode & kOwnCodes) ? 256 : 2 * 256;
+}
+struct PairTabs {
+    const uint32_t* M;
+    const float *Mf, *QW, *QWc;
+    const int32_t *QWi, *Q, *W;
+};
+// Views of a table part that starts at byte pair_tab_first(MODE) of its set.
+template <unsigned MODE>
+__device__ __forceinline__ PairTabs pair_tabs(const uint8_t* part) {
+    PairTabs t{};
+    if (MODE & kLoadPix) {
+        t.M = reinterpret_cast<const uint32_t*>(part);
+        t.Mf = reinterpret_cast<const float*>(part + 256);
+        t.QW = reinterpret_cast<const float*>(part + 512);
+        t.QWc = reinterpret_cast<const float*>(part + 768);
+    } else if (MODE & kOwnCodes) {
+        t.QWi = reinterpret_cast<const int32_t*>(part);
+    } else {
+        t.Q = reinterpret_cast<const int32_t*>(part);
+        t.W = reinterpret_cast<const int32_t*>(part + 256);
+    }
+    return t;
 }
 
-// The two-lane tile implements the fused modes (samples in, inverse out),
-// the forward pass alone (samples in, coefficients out) and the inverse pass
-// alone (coefficients in, reconstruction and/or SSE out); the statistics
-// modes keep the one-lane tile.
+// Shared memory per warp of the two-lane batched kernel: tables, descriptor,
+// transpose buffer, sample slots.
+__host__ __device__ constexpr int pair_warp_smem_bytes(unsigned mode) {
+    return pair_tab_bytes(mode) + kDescBytes + kXBytes + kParkBytes;
+}
+
+// The two-lane tile implements the fused modes (samples in, inverse out) and
+// the inverse pass alone (coefficients in, reconstruction and/or SSE out); the
+// forward pass alone and the statistics modes keep the one-lane tile.
 __host__ __device__ constexpr bool pair_mode_supported(unsigned mode) {
-    return !(mode & (kStats | kStatsPrivate)) &&
-           (((mode & kLoadPix) && !(mode & kLoadCoef) && ((mode & kInverse) || mode == (kLoadPix | kStoreCoef))) ||
-            ((mode & kLoadCoef) && (mode & kInverse) && !(mode & (kLoadPix | kStoreCoef))));
+    return !(mode & (kStats | kStatsPrivate)) && (mode & kInverse) && !(mode & kLoadPix) == !!(mode & kLoadCoef) &&
+           !((mode & kLoadCoef) && (mode & kStoreCoef));
 }
 
 // Loads rows 4h..4h+3 of block (by, bx) as two little-endian words each,
@@ -123,24 +158,44 @@ __device__ __forceinline__ void unpark_rows(const uint8_t* slot, int sw, uint32_
     pix[2][0] = b.x; pix[2][1] = b.y; pix[3][0] = b.z; pix[3][1] = b.w;
 }
 
-// Processes warp tile `tile_in_plane` of plane P (two half tiles of 16
-// blocks).  xb is this warp's kXBytes transpose buffer followed by its
-// kParkBytes sample slots.  Returns the tile's SSE (the same in every lane;
-// 0 without kSse).
+// Rows U.. of a lane's four columns: quantised codes to the stage at xc and,
+// for the fused modes, dequantised inputs of the inverse column pass.
+template <unsigned MODE, bool FLT, int U = 0>
+__device__ __forceinline__ void pair_quant_rows(const PairTabs& T, int h, uint8_t* xc, int sw, const float (&y)[4][8],
+                                                int (&c)[4][8]) {
+    if constexpr (U < 8) {
+        const float4 mf = *reinterpret_cast<const float4*>(&T.Mf[4 * h + U * 8]);
+        const float t0 = quant_code<FLT, U, 0>(y[0][U], mf.x, T.M + 4 * h);
+        const float t1 = quant_code<FLT, U, 1>(y[1][U], mf.y, T.M + 4 * h);
+        const float t2 = quant_code<FLT, U, 2>(y[2][U], mf.z, T.M + 4 * h);
+        const float t3 = quant_code<FLT, U, 3>(y[3][U], mf.w, T.M + 4 * h);
+        if (MODE & kStoreCoef)
+            *reinterpret_cast<uint2*>(xc + ((U ^ sw) << 4)) = make_uint2(pack_codes(t0, t1), pack_codes(t2, t3));
+        if (MODE & kInverse) {
+            const float4 qw = *reinterpret_cast<const float4*>(&T.QW[4 * h + U * 8]);
+            const float4 qc = *reinterpret_cast<const float4*>(&T.QWc[4 * h + U * 8]);
+            c[0][U] = dequant_bits(t0, qw.x, qc.x);
+            c[1][U] = dequant_bits(t1, qw.y, qc.y);
+            c[2][U] = dequant_bits(t2, qw.z, qc.z);
+            c[3][U] = dequant_bits(t3, qw.w, qc.w);
+        }
+        pair_quant_rows<MODE, FLT, U + 1>(T, h, xc, sw, y, c);
+    }
+}
+
+// Processes halves hf0..hf1 - 1 (16 blocks each) of warp tile `tile_in_plane`
+// of plane P.  xb is this warp's kXBytes transpose buffer followed by its
+// kParkBytes sample slots.  Returns their SSE (the same in every lane; 0
+// without kSse).
 template <unsigned MODE>
-__device__ __forceinline__ unsigned process_tile_pair(const PlaneArg& P, const QuantSet& T, int tile_in_plane,
-                                                      int lane, uint8_t* xb) {
+__device__ __forceinline__ unsigned process_tile_pair(const PlaneArg& P, const PairTabs& T, int tile_in_plane,
+                                                      int lane, uint8_t* xb, int hf0 = 0, int hf1 = 2) {
     static_assert(pair_mode_supported(MODE), "no two-lane form of this mode");
     const int k = lane >> 1, h = lane & 1;
     uint8_t* const xw = xb + k * kXSlot + h * kXRowHalf;   // rows 4h..4h+3, both quads
     uint8_t* const xr = xb + k * kXSlot + h * 16;           // rows 0..7, quad h
-    // descale rounding term and +128 level, added once to the DC input
-    // (column 0 belongs to lane h = 0)
-    const int dc_bias = h ? 0 : (1 << (kR + 2)) + (128 << (kR + 3));
-    const int32_t* Mh = reinterpret_cast<const int32_t*>(T.M) + 4 * h;
-    const int32_t* QWh = T.QW + 4 * h;
-    const int32_t* Qh = T.Q + 4 * h;
-    const int32_t* Wh = T.W + 4 * h;
+    // the DC input (column 0) belongs to lane h = 0
+    const int dc_bias = h ? 0 : kDcBias;
     uint8_t* const park = xb + kXBytes + lane * 32;
     const int psw = (lane >> 2) & 1;
     unsigned e = 0;
@@ -150,7 +205,7 @@ __device__ __forceinline__ unsigned process_tile_pair(const PlaneArg& P, const Q
     const int bx_t = bt - by_t * P.nbx;
 
 #pragma unroll 1
-    for (int hf = 0; hf < 2; ++hf) {
+    for (int hf = hf0; hf < hf1; ++hf) {
         const int b0 = bt + hf * kPairBlocks;
         const int nvalid = min(kPairBlocks, P.nblk - b0);
         if (nvalid <= 0) break;                      // warp-uniform
@@ -169,19 +224,17 @@ __device__ __forceinline__ unsigned process_tile_pair(const PlaneArg& P, const Q
         int c[4][8];
         uint32_t pix[4][2];
         if (MODE & kLoadPix) {
-            // level shift and row pass on rows 4h..4h+3
+            // row pass on rows 4h..4h+3
             if (active) {
                 load_rows4(P.src, P.src_pitch, P.width, P.height, by, bx, h, (P.flags & kVecSrc) != 0, pix);
             } else {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) pix[j][0] = pix[j][1] = 0x80808080u;
             }
+            float z[4][8];
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-#pragma unroll
-                for (int col = 0; col < 8; ++col) v[j][col] = (sample4(pix, j, col) - 128) * (1 << kP);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) loeffler8_fwd<false>(v[j]);
+            for (int j = 0; j < 4; ++j) pix_row(pix[j], z[j]);
+            fwd_vectors<true>(z);
 
             // the samples wait for the SSE in this lane's slot (the two 16-byte
             // halves swap on every fourth lane: no bank conflicts)
@@ -191,56 +244,38 @@ __device__ __forceinline__ unsigned process_tile_pair(const PlaneArg& P, const Q
             __syncwarp();
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                sts128(xw + j * 32, v[j][0], v[j][1], v[j][2], v[j][3]);
-                sts128(xw + j * 32 + 16, v[j][4], v[j][5], v[j][6], v[j][7]);
+                *reinterpret_cast<float4*>(xw + j * 32) = make_float4(z[j][0], z[j][1], z[j][2], z[j][3]);
+                *reinterpret_cast<float4*>(xw + j * 32 + 16) = make_float4(z[j][4], z[j][5], z[j][6], z[j][7]);
             }
             __syncwarp();
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
-                const int4 t = lds128(xr + (r >> 2) * kXRowHalf + (r & 3) * 32);
-                c[0][r] = t.x;
-                c[1][r] = t.y;
-                c[2][r] = t.z;
-                c[3][r] = t.w;
+                const float4 t = *reinterpret_cast<const float4*>(xr + (r >> 2) * kXRowHalf + (r & 3) * 32);
+                z[0][r] = t.x;
+                z[1][r] = t.y;
+                z[2][r] = t.z;
+                z[3][r] = t.w;
             }
 
-            // column pass: c[i][u] = Y[u][4h + i]
-#pragma unroll
-            for (int i = 0; i < 4; ++i) loeffler8_fwd<false>(c[i]);
+            // column pass: z[i][u] = Y[u][4h + i]
+            fwd_vectors<false>(z);
 
-            // quantiser: high word of Y M + 2^31, with - [Y < 0] at the tie
-            // entries (u, v in {0, 4}: i = 0 and u = 0 or 4 in both lanes)
+            // quantiser and own-code dequantiser; the codes go through the
+            // transpose buffer (free between the two transposes) so that the
+            // stores to global memory move 512 contiguous bytes each
+            if (MODE & kStoreCoef) __syncwarp();             // transpose reads done
+            uint8_t* const xc = xb + k * 128 + h * 8;
+            if (T.Mf[0] != 0.0f) pair_quant_rows<MODE, true>(T, h, xc, k & 7, z, c);
+            else pair_quant_rows<MODE, false>(T, h, xc, k & 7, z, c);
+            if (MODE & kStoreCoef) {
+                __syncwarp();
+                uint4* const g = reinterpret_cast<uint4*>(P.coef + (size_t)b0 * 64) + lane;
+                const uint8_t* const xs = xb + (lane >> 3) * 128;
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int4 m = *reinterpret_cast<const int4*>(Mh + u * 8);
-                const int mv[4] = {m.x, m.y, m.z, m.w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int y = c[i][u];
-                    long long p = (long long)y * (long long)mv[i] + 0x80000000ll;
-                    if (tie_entry(u, i)) p += (long long)(y >> 31);
-                    c[i][u] = (int)(p >> 32);
-                }
-            }
-
-            // coefficients: row u of the block is 16 bytes, lane h writes its half
-            if ((MODE & kStoreCoef) && active) {
-                uint2* g = reinterpret_cast<uint2*>(P.coef + (size_t)(b0 + k) * 64 + 4 * h);
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    g[2 * u] = make_uint2(((uint32_t)c[0][u] & 0xFFFFu) | ((uint32_t)c[1][u] << 16),
-                                          ((uint32_t)c[2][u] & 0xFFFFu) | ((uint32_t)c[3][u] << 16));
-            }
-            // dequantiser G = q (Q W): the clamp of the definition never acts
-            // on this kernel's own codes (|q Q| < 1200)
-            if (MODE & kInverse) {
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int4 qw = *reinterpret_cast<const int4*>(QWh + u * 8);
-                    c[0][u] *= qw.x;
-                    c[1][u] *= qw.y;
-                    c[2][u] *= qw.z;
-                    c[3][u] *= qw.w;
+                for (int i = 0; i < 4; ++i) {                // chunk 32 i + lane: block 4 i + lane / 8, row lane % 8
+                    const uint4 w = *reinterpret_cast<const uint4*>(
+                        xs + i * 512 + (((lane & 7) ^ ((4 * i + (lane >> 3)) & 7)) << 4));
+                    if (4 * i + (lane >> 3) < nvalid) g[32 * i] = w;
                 }
             }
         } else {
@@ -269,7 +304,7 @@ __device__ __forceinline__ unsigned process_tile_pair(const PlaneArg& P, const Q
                 // clamp never acts (|q Q| < 1200)
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
-                    const int4 qw = *reinterpret_cast<const int4*>(QWh + u * 8);
+                    const int4 qw = *reinterpret_cast<const int4*>(T.QWi + 4 * h + u * 8);
                     c[0][u] *= qw.x;
                     c[1][u] *= qw.y;
                     c[2][u] *= qw.z;
@@ -279,8 +314,8 @@ __device__ __forceinline__ unsigned process_tile_pair(const PlaneArg& P, const Q
                 // dequantiser G = clamp(q Q, -4096, 4096) W for arbitrary codes
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
-                    const int4 q4 = *reinterpret_cast<const int4*>(Qh + u * 8);
-                    const int4 w4 = *reinterpret_cast<const int4*>(Wh + u * 8);
+                    const int4 q4 = *reinterpret_cast<const int4*>(T.Q + 4 * h + u * 8);
+                    const int4 w4 = *reinterpret_cast<const int4*>(T.W + 4 * h + u * 8);
                     c[0][u] = max(-kDequantClamp, min(kDequantClamp, c[0][u] * q4.x)) * w4.x;
                     c[1][u] = max(-kDequantClamp, min(kDequantClamp, c[1][u] * q4.y)) * w4.y;
                     c[2][u] = max(-kDequantClamp, min(kDequantClamp, c[2][u] * q4.z)) * w4.z;
@@ -289,11 +324,10 @@ __device__ __forceinline__ unsigned process_tile_pair(const PlaneArg& P, const Q
             }
         }
         if constexpr ((MODE & kInverse) != 0) {
-            c[0][0] += dc_bias;
-
             // inverse column pass, transpose back, inverse row pass
+            constexpr int Z = (MODE & kLoadPix) ? kMagicBits : 0;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) loeffler8_inv(c[i]);
+            for (int i = 0; i < 4; ++i) loeffler8_inv<Z>(c[i], i == 0 ? dc_bias : 0);
             __syncwarp();                                // transpose reads done
 #pragma unroll
             for (int r = 0; r < 8; ++r)
@@ -307,23 +341,11 @@ __device__ __forceinline__ unsigned process_tile_pair(const PlaneArg& P, const Q
                 v[j][4] = b.x; v[j][5] = b.y; v[j][6] = b.z; v[j][7] = b.w;
             }
 #pragma unroll
-            for (int j = 0; j < 4; ++j) loeffler8_inv(v[j]);
+            for (int j = 0; j < 4; ++j) loeffler8_inv<0>(v[j], 0);
 
-            // descale, clamp, pack
             uint32_t out[4][2];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    uint32_t wd = 0;
-#pragma unroll
-                    for (int t = 0; t < 4; ++t) {
-                        const int s = clamp_u8(v[j][4 * q + t] >> (kR + 3));
-                        wd |= (uint32_t)s << (8 * t);
-                    }
-                    out[j][q] = wd;
-                }
-            }
+            for (int j = 0; j < 4; ++j) descale_row(v[j], out[j]);
             if ((MODE & kStoreRecon) && active)
                 store_rows4(P.dst, P.dst_pitch, P.width, P.height, by, bx, h, (P.flags & kVecDst) != 0, out);
 
@@ -351,8 +373,8 @@ __device__ __forceinline__ unsigned process_tile_pair(const PlaneArg& P, const Q
     return (MODE & kSse) ? warp_sum(e) : 0u;
 }
 
-// Direct (non-batched) fused calls with two lanes per block: grid-stride over
-// the warp tiles of up to kMaxPlanes planes, tables in shared memory, SSE
+// Direct (non-batched) calls with two lanes per block: grid-stride over the
+// half tiles of up to kMaxPlanes planes, tables in shared memory, SSE
 // summed per CTA and added to each plane's word once (zero on entry).
 constexpr int kPairCodecHeader = 2 * (int)sizeof(QuantSet) + kMaxPlanes * 8;
 static_assert(kPairCodecHeader % 16 == 0, "per-warp buffers must stay 16-byte aligned");
@@ -367,23 +389,23 @@ __global__ void __launch_bounds__(256, DCTGB_PAIR_MINB) k_codec_pair(const __gri
     QuantSet* tabs = reinterpret_cast<QuantSet*>(smem);
     unsigned long long* csse = reinterpret_cast<unsigned long long*>(smem + 2 * sizeof(QuantSet));
     {
-        const uint32_t* s = reinterpret_cast<const uint32_t*>(args.tabs);
-        uint32_t* d = reinterpret_cast<uint32_t*>(tabs);
-        for (int i = threadIdx.x; i < (int)(2 * sizeof(QuantSet) / 4); i += blockDim.x) d[i] = s[i];
         if (threadIdx.x < kMaxPlanes) csse[threadIdx.x] = 0ull;
-        __syncthreads();
+        build_tabs(args.tabs, tabs);
     }
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int warps_per_cta = blockDim.x >> 5;
     uint8_t* xb = smem + kPairCodecHeader + warp * (kXBytes + kParkBytes);
-    for (int tile = blockIdx.x * warps_per_cta + warp; tile < args.ntiles; tile += gridDim.x * warps_per_cta) {
+    for (int unit = blockIdx.x * warps_per_cta + warp; unit < 2 * args.ntiles; unit += gridDim.x * warps_per_cta) {
+        const int tile = unit >> 1, hf = unit & 1;
         int pi = 0;
 #pragma unroll
         for (int k = 1; k < kMaxPlanes; ++k)
             if (k < args.nplanes && tile >= args.p[k].tile_begin) pi = k;
         const PlaneArg& P = args.p[pi];
-        const unsigned e = process_tile_pair<MODE>(P, tabs[P.table], tile - P.tile_begin, lane, xb);
+        const uint8_t* part = reinterpret_cast<const uint8_t*>(&tabs[P.table]) + pair_tab_first(MODE);
+        const unsigned e = process_tile_pair<MODE>(P, pair_tabs<MODE>(part), tile - P.tile_begin, lane, xb,
+                                                       hf, hf + 1);
         if ((MODE & kSse) && lane == 0 && e) atomicAdd(&csse[pi], (unsigned long long)e);
     }
     __syncthreads();
@@ -391,21 +413,22 @@ __global__ void __launch_bounds__(256, DCTGB_PAIR_MINB) k_codec_pair(const __gri
         atomicAdd(args.p[threadIdx.x].sse, csse[threadIdx.x]);
 }
 
-// Host launcher of k_codec_pair: one persistent grid of resident CTAs.  A
-// call with fewer tiles than warps in `num_sms` CTAs of `threads` gets
+// Host launcher of k_codec_pair: one grid of resident CTAs (direct_grid).  A
+// call with fewer half tiles than warps in `num_sms` CTAs of `threads` gets
 // smaller CTAs (down to two warps), so a small plane spreads over more SMs
-// instead of sharing a few SMs' schedulers (a tile takes one warp many
-// microseconds, so that sharing sets the latency of the whole call).
+// instead of sharing a few SMs' schedulers (a half tile takes one warp
+// several microseconds, so that sharing sets the latency of the whole call).
 template <unsigned MODE>
 inline cudaError_t launch_codec_pair(const DirectArgs& a, int num_sms, int threads, cudaStream_t s) {
-    while (threads > 64 && (long long)a.ntiles < (long long)num_sms * (threads / 32)) threads /= 2;
+    const int units = 2 * a.ntiles;
+    while (threads > 64 && (long long)units < (long long)num_sms * (threads / 32)) threads /= 2;
     const size_t smem = pair_codec_smem_bytes(threads);
     cudaError_t e = cudaFuncSetAttribute(k_codec_pair<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int occ = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_codec_pair<MODE>, threads, smem);
     if (e != cudaSuccess) return e;
-    k_codec_pair<MODE><<<persistent_grid(a.ntiles, threads, num_sms, occ), threads, smem, s>>>(a);
+    k_codec_pair<MODE><<<direct_grid(units, threads, num_sms, occ), threads, smem, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -37,7 +37,7 @@ constexpr int kRgbSmem = 2 * (int)sizeof(QuantSet) + kRgbYBytes + 2 * kRgbCBytes
 struct RgbArgs {
     const uint8_t* rgb;
     int16_t* coef;                 // Y codes, then Cb, then Cr (dct_compress layout)
-    QuantSet tabs[2];              // luma, chroma
+    TabArgs tabs;                  // luma, chroma
     int32_t width, height, pitch;  // pixels, bytes between RGB rows
     int32_t cw, ch;                // chroma plane size
     int32_t nbx_y, nby_y;          // luma block grid
@@ -53,27 +53,6 @@ __device__ __forceinline__ void rgb_convert(const uint8_t* p, int& y, int& cb, i
     cr = max(0, min(255, (32768 * r - 27439 * g - 5329 * b + (128 << 16) + 32768) >> 16));
 }
 
-// Forward-path quantiser of the one-lane tile: the high word of Y M + 2^31
-// away from the four tie entries, |Y| with an unsigned multiply and the sign
-// there (tie_entry).
-__device__ __forceinline__ void quantize_fwd(int (&x)[8][8], const QuantSet& T) {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-#pragma unroll
-        for (int v = 0; v < 8; ++v) {
-            const int y = x[u][v];
-            if (!tie_entry(u, v)) {
-                const long long p = (long long)y * (long long)(int)T.M[u * 8 + v] + 0x80000000ll;
-                x[u][v] = (int)(p >> 32);
-            } else {
-                const uint32_t a = (uint32_t)abs(y);
-                const uint32_t q = (uint32_t)(((unsigned long long)a * T.M[u * 8 + v] + 0x80000000ull) >> 32);
-                x[u][v] = y < 0 ? -(int)q : (int)q;
-            }
-        }
-    }
-}
-
 __global__ void __launch_bounds__(kRgbThreads, 6) k_compress_rgb(const __grid_constant__ RgbArgs a) {
     extern __shared__ __align__(16) uint8_t smem[];
     QuantSet* tabs = reinterpret_cast<QuantSet*>(smem);
@@ -83,11 +62,7 @@ __global__ void __launch_bounds__(kRgbThreads, 6) k_compress_rgb(const __grid_co
     uint8_t* stage = crs + kRgbCBytes;                    // [96][128]
     uint8_t* raw = stage + kRgbThreads * 128;             // [16][kRgbRawRow] RGB bytes of the strip
     int* lead16 = reinterpret_cast<int*>(raw + 16 * kRgbRawRow);   // [16] offset of each row in its chunk
-    {
-        const uint32_t* s = reinterpret_cast<const uint32_t*>(a.tabs);
-        uint32_t* d = reinterpret_cast<uint32_t*>(tabs);
-        for (int i = threadIdx.x; i < (int)(2 * sizeof(QuantSet) / 4); i += blockDim.x) d[i] = s[i];
-    }
+    build_tabs(a.tabs, tabs);
     const int t = threadIdx.x;
     for (int unit = blockIdx.x; unit < a.units; unit += gridDim.x) {
         const int my = unit / a.units_x;
@@ -174,25 +149,25 @@ __global__ void __launch_bounds__(kRgbThreads, 6) k_compress_rgb(const __grid_co
         const int spitch = luma ? kRgbUnitW : kRgbUnitW / 2;
         const bool valid = luma ? (2 * my + (t >> 5) < a.nby_y && 2 * mx0 + k < a.nbx_y) : (mx0 + k < a.nbx_c);
         if (valid) {
-            int x[8][8];
+            uint32_t pix[8][2];
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
                 const uint2 w = *reinterpret_cast<const uint2*>(src + r * spitch);
-#pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    x[r][c] = ((int)(((c < 4 ? w.x : w.y) >> (8 * (c & 3))) & 0xFFu) - 128) * (1 << kP);
+                pix[r][0] = w.x;
+                pix[r][1] = w.y;
             }
-            fwd2d<false>(x);
-            quantize_fwd(x, tabs[luma ? 0 : 1]);
+            float f[8][8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                uint4 w;
-                w.x = ((uint32_t)x[u][0] & 0xFFFFu) | ((uint32_t)x[u][1] << 16);
-                w.y = ((uint32_t)x[u][2] & 0xFFFFu) | ((uint32_t)x[u][3] << 16);
-                w.z = ((uint32_t)x[u][4] & 0xFFFFu) | ((uint32_t)x[u][5] << 16);
-                w.w = ((uint32_t)x[u][6] & 0xFFFFu) | ((uint32_t)x[u][7] << 16);
-                *reinterpret_cast<uint4*>(stage + t * 128 + ((u ^ (t & 7)) << 4)) = w;
-            }
+            for (int r = 0; r < 8; ++r) pix_row(pix[r], f[r]);
+            fwd_vectors<true>(f);
+            const QuantSet& T = tabs[luma ? 0 : 1];
+            unsigned ac = 0;
+            uint32_t w[8][4];
+            int x[8][8];
+            fwd_columns<kStoreCoef>(T, f, true, 0, nullptr, ac, w, x);
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                *reinterpret_cast<uint4*>(stage + t * 128 + ((u ^ (t & 7)) << 4)) = make_uint4(w[u][0], w[u][1], w[u][2], w[u][3]);
         }
         __syncthreads();
 
@@ -237,8 +212,7 @@ extern "C" dct_status dct_compress_rgb(dct_plan_t plan, const uint8_t* rgb, int3
     if (((uintptr_t)coeffs) & 15u) return fail(DCT_ERR_INVALID_ARG, "coeffs must be 16-byte aligned");
     RgbArgs a;
     memset(&a, 0, sizeof a);
-    dct_status st = build_tables(quality, qtab_host, qtab_entries, 0, a.tabs[0]);
-    if (st == DCT_OK) st = build_tables(quality, qtab_host, qtab_entries, 1, a.tabs[1]);
+    dct_status st = build_tab_args(quality, qtab_host, qtab_entries, true, a.tabs);
     if (st != DCT_OK) return st;
     a.rgb = rgb;
     a.coef = coeffs;
