@@ -1,7 +1,8 @@
 """The arithmetic forms the kernels use in place of the definitions, re-derived
 on the CPU: the quantiser and the own-code dequantiser as one float32 fused
-multiply-add each, and the first two micro-rotations of the row pass as one
-linear map.  A GPU case runs tables that mix entries with and
+multiply-add each, the first two micro-rotations of the row pass as one linear
+map, and the transposed rotations on signed, offset operands (one shift-add
+per half micro-rotation).  A GPU case runs tables that mix entries with and
 without an exact float multiplier through every forward entry point."""
 import numpy as np
 import pytest
@@ -70,6 +71,50 @@ def test_row_pass_steps_1_and_2_are_linear(n):
         x, y = cl.cordic_rotate(a, b, sig[:2])
         c, k = 1 - sig[0] * sig[1] / 8, sig[0] / 2 + sig[1] / 4
         assert np.array_equal(x, a * c + b * k) and np.array_equal(y, b * c - a * k)
+
+
+def offset_run(sig, ka, kb, upto):
+    """Offsets and signs after `upto` transposed steps from (+a + ka, +b + kb); None when a shift is not exact."""
+    sa = sb = 1
+    for i in range(1, upto + 1):
+        s, m = -sig[i - 1], 1 << i
+        if (kb if sb > 0 else kb + 1) % m or (ka if sa > 0 else ka + 1) % m:
+            return None
+        cb = kb // m if sb > 0 else (kb + 1) // m - 1
+        ca = ka // m if sa > 0 else (ka + 1) // m - 1
+        fa, fb = sb != sa * s, sa != -s * sb
+        ka, kb = (-ka if fa else ka) + cb, (-kb if fb else kb) + ca
+        sa, sb = (-sa if fa else sa), (-sb if fb else sb)
+    return ka, kb, sa, sb
+
+
+@pytest.mark.parametrize("n", NS)
+@pytest.mark.parametrize("name", ["odd_upper", "odd_lower", "even"])
+def test_offset_rotation_equals_the_transposed_rotation(n, name):
+    sig = getattr(cl.Sigmas(n), name)
+    ka = kb = bits = 0
+    for i in range(1, n + 1):                                # lift the starting offsets step by step
+        sol = [(x, y) for x in range(1 << i) for y in range(1 << i)
+               if offset_run(sig, ka + (x << bits), kb + (y << bits), i) is not None]
+        assert len(sol) == 1                                 # exactly one solution modulo 2^(1 + .. + i)
+        ka, kb, bits = ka + (sol[0][0] << bits), kb + (sol[0][1] << bits), bits + i
+    m = 1 << bits
+    ka, kb = (ka - m if ka >= m // 2 else ka), (kb - m if kb >= m // 2 else kb)
+    eka, ekb, esa, esb = offset_run(sig, ka, kb, n)
+    assert max(map(abs, (ka, kb, eka, ekb))) < 1 << 22       # nodes below 1.17e9 leave room in int32
+    rng = np.random.default_rng(10 * n)
+    lim = 1 << 29
+    a = np.concatenate([rng.integers(-lim, lim, 5000), rng.integers(-70, 71, 5000), [-lim, lim, 0, -1, 1]])
+    b = np.concatenate([rng.integers(-lim, lim, 5000), rng.integers(-70, 71, 5000), [lim, -lim, 0, 1, -1]])
+    A, B, sa, sb = a + ka, b + kb, 1, 1
+    for i in range(1, n + 1):
+        s = -sig[i - 1]
+        fa, fb = sb != sa * s, sa != -s * sb
+        A, B = ((B >> i) - A if fa else A + (B >> i)), ((A >> i) - B if fb else B + (A >> i))
+        assert max(np.abs(A).max(), np.abs(B).max()) < 1 << 31
+        sa, sb = (-sa if fa else sa), (-sb if fb else sb)
+    wa, wb = cl.cordic_rotate_t(a, b, sig)
+    assert np.array_equal(A, esa * wa + eka) and np.array_equal(B, esb * wb + ekb)
 
 
 @pytest.mark.gpu
