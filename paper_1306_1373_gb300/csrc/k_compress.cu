@@ -14,8 +14,8 @@ static cudaError_t launch_mode(const DirectArgs& a, int num_sms, int threads, cu
     int occ = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_codec<MODE>, threads, smem);
     if (e != cudaSuccess) return e;
-    k_codec<MODE><<<direct_grid(a.ntiles, threads, num_sms, occ), threads, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_behind_init(k_codec<MODE>, direct_grid(a.ntiles, threads, num_sms, occ), threads, smem, s, a,
+                              (MODE & kStats) != 0);
 }
 
 cudaError_t launch_compress(const DirectArgs& a, bool stats, int num_sms, int threads, cudaStream_t s) {
@@ -24,6 +24,7 @@ cudaError_t launch_compress(const DirectArgs& a, bool stats, int num_sms, int th
 }
 
 __global__ void k_init_acc(DirectArgs args, int do_sse, int do_stats) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (int pl = 0; pl < args.nplanes; ++pl) {
         if (do_sse && threadIdx.x == 0) *args.p[pl].sse = 0ull;
         if (do_stats)

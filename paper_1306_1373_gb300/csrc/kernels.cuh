@@ -115,8 +115,8 @@ constexpr uint32_t kTieFreeBits = 0xFFFu;   // (M & kTieFreeBits) != 0  <=>  k <
 
 // The float multiplier of M (above): false when M needs more than 24 bits.
 __host__ __device__ inline bool quant_multiplier(uint32_t m, float& out) {
+    if ((m >> 24) && (m & ((2u << (m >> 25 ? (m >> 26 ? 2 : 1) : 0)) - 1u))) return false;   // M < 2^27
     const float f = (float)m;
-    if ((double)f != (double)m) return false;
     out = f * 2.3283064365386963e-10f;      // 2^-32
     if ((m & kTieFreeBits) == 0) {          // the next float above
         union { float f; uint32_t u; } b;
@@ -233,6 +233,50 @@ __device__ __forceinline__ bool interior(const PlaneArg& P, int by, int bx) {
     return bx * 8 + 8 <= P.width && by * 8 + 8 <= P.height;
 }
 
+// Eight bytes from any address, as aligned words and funnel shifts: three
+// loads instead of eight (a plane with tight odd rows was bound by its byte
+// accesses: 64 loads and 64 stores per block).  The words that hold the bytes
+// must lie in the plane.
+__device__ __forceinline__ void load8_unaligned(const uint8_t* p, uint32_t (&w)[2]) {
+    const unsigned o = (unsigned)(uintptr_t)p & 3u;
+    const uint32_t* q = reinterpret_cast<const uint32_t*>(p - o);
+    const uint32_t a = __ldg(q), b = __ldg(q + 1), c = o ? __ldg(q + 2) : 0u;
+    w[0] = __funnelshift_r(a, b, 8 * o);
+    w[1] = __funnelshift_r(b, c, 8 * o);
+}
+// Whether load8_unaligned may read rows y0..y1 at column x0: its words then
+// start at or after the plane's first byte and end at or before its last.
+__device__ __forceinline__ bool words_inside(const uint8_t* src, int pitch, int w, int h, int y0, int y1, int x0) {
+    const uintptr_t first = (uintptr_t)src, last = first + (size_t)(h - 1) * pitch + w;
+    return (((uintptr_t)(src + (size_t)y0 * pitch + x0)) & ~(uintptr_t)3) >= first &&
+           (((uintptr_t)(src + (size_t)y1 * pitch + x0 + 8) + 3) & ~(uintptr_t)3) <= last;
+}
+
+// Eight bytes to any address, as the widest aligned stores that cover them.
+__device__ __forceinline__ void store8_unaligned(uint8_t* p, const uint32_t (&w)[2]) {
+    const unsigned o = (unsigned)(uintptr_t)p & 3u;
+    if (o == 0) {
+        reinterpret_cast<uint32_t*>(p)[0] = w[0];
+        reinterpret_cast<uint32_t*>(p)[1] = w[1];
+    } else if (o == 2) {
+        *reinterpret_cast<uint16_t*>(p) = (uint16_t)w[0];
+        *reinterpret_cast<uint32_t*>(p + 2) = __funnelshift_r(w[0], w[1], 16);
+        *reinterpret_cast<uint16_t*>(p + 6) = (uint16_t)(w[1] >> 16);
+    } else {
+        // one byte, then 2 + 4 bytes (o = 1) or 4 + 2 bytes (o = 3), one byte
+        p[0] = (uint8_t)w[0];
+        p[7] = (uint8_t)(w[1] >> 24);
+        const uint32_t lo = __funnelshift_r(w[0], w[1], 8);          // bytes 1..4
+        if (o == 1) {
+            *reinterpret_cast<uint16_t*>(p + 1) = (uint16_t)lo;
+            *reinterpret_cast<uint32_t*>(p + 3) = __funnelshift_r(w[0], w[1], 24);
+        } else {
+            *reinterpret_cast<uint32_t*>(p + 1) = lo;
+            *reinterpret_cast<uint16_t*>(p + 5) = (uint16_t)(w[1] >> 8);
+        }
+    }
+}
+
 // Loads block (by, bx) as 8 rows of two little-endian uint32 words.  Samples
 // outside the plane repeat the nearest edge sample (edge replication).
 __device__ __forceinline__ void load_block(const uint8_t* __restrict__ src, int pitch, int w, int h,
@@ -246,6 +290,10 @@ __device__ __forceinline__ void load_block(const uint8_t* __restrict__ src, int 
             pix[r][0] = v.x;
             pix[r][1] = v.y;
         }
+    } else if (x0 + 8 <= w && y0 + 8 <= h && words_inside(src, pitch, w, h, y0, y0 + 7, x0)) {
+        const uint8_t* p = src + (size_t)y0 * pitch + x0;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) load8_unaligned(p + (size_t)r * pitch, pix[r]);
     } else {
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
@@ -317,6 +365,10 @@ __device__ __forceinline__ void store_block(uint8_t* __restrict__ dst, int pitch
 #pragma unroll
         for (int r = 0; r < 8; ++r)
             *reinterpret_cast<uint2*>(p + (size_t)r * pitch) = make_uint2(pix[r][0], pix[r][1]);
+    } else if (x0 + 8 <= w && y0 + 8 <= h) {
+        uint8_t* p = dst + (size_t)y0 * pitch + x0;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) store8_unaligned(p + (size_t)r * pitch, pix[r]);
     } else {
         const int nr = min(8, h - y0), nc = min(8, w - x0);
         for (int r = 0; r < nr; ++r) {
@@ -658,6 +710,14 @@ __device__ __forceinline__ unsigned process_tile(const PlaneArg& P, const QuantS
 // persistent kernel over all tiles of up to kMaxPlanes planes (direct calls)
 // --------------------------------------------------------------------------
 
+// The kernel behind k_init_acc may start while it still runs (a programmatic
+// dependent launch: k_init_acc lets its dependents go at once, so everything
+// before it in the stream has finished) and waits for it only where it adds to
+// the cleared words, at its end.  The clearing launch takes about 3 us by
+// itself; 2731 x 1823 fused with unaligned rows: 18.4 us a call with it hidden
+// and rows read as words, 20.5 us before.
+__device__ __forceinline__ void init_acc_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 struct CtaAcc {
     unsigned long long sse[kMaxPlanes];
     unsigned long long st[kMaxPlanes][kStatsWords];
@@ -699,6 +759,7 @@ __global__ void __launch_bounds__(256, DCTGB_MINB) k_codec(const __grid_constant
     }
 
     __syncthreads();
+    if (MODE & (kSse | kStats)) init_acc_wait();
     if (MODE & kSse) {
         if (threadIdx.x < args.nplanes && acc->sse[threadIdx.x])
             atomicAdd(args.p[threadIdx.x].sse, acc->sse[threadIdx.x]);
@@ -721,6 +782,22 @@ __global__ void __launch_bounds__(256, DCTGB_MINB) k_codec(const __grid_constant
 
 // zero the SSE words and the statistics (min words to all ones)
 __global__ void k_init_acc(DirectArgs args, int do_sse, int do_stats);
+
+template <typename Args>
+inline cudaError_t launch_behind_init(void (*kernel)(Args), int grid, int threads, size_t smem, cudaStream_t s,
+                                      const Args& a, bool init) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = init ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, a);
+}
 
 inline size_t codec_smem_bytes(int threads) {
     return 2 * sizeof(QuantSet) + sizeof(CtaAcc) + (size_t)(threads / 32) * kStageBytes;

@@ -101,6 +101,10 @@ __device__ __forceinline__ void load_rows4(const uint8_t* __restrict__ src, int 
             pix[j][0] = v.x;
             pix[j][1] = v.y;
         }
+    } else if (x0 + 8 <= w && by * 8 + 8 <= hgt && words_inside(src, pitch, w, hgt, y0, y0 + 3, x0)) {
+        const uint8_t* p = src + (size_t)y0 * pitch + x0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) load8_unaligned(p + (size_t)j * pitch, pix[j]);
     } else {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -127,6 +131,10 @@ __device__ __forceinline__ void store_rows4(uint8_t* __restrict__ dst, int pitch
 #pragma unroll
         for (int j = 0; j < 4; ++j)
             *reinterpret_cast<uint2*>(p + (size_t)j * pitch) = make_uint2(pix[j][0], pix[j][1]);
+    } else if (x0 + 8 <= w && by * 8 + 8 <= hgt) {
+        uint8_t* p = dst + (size_t)y0 * pitch + x0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) store8_unaligned(p + (size_t)j * pitch, pix[j]);
     } else {
         const int nr = min(4, hgt - y0), nc = min(8, w - x0);
         for (int j = 0; j < nr; ++j) {
@@ -409,6 +417,7 @@ __global__ void __launch_bounds__(256, DCTGB_PAIR_MINB) k_codec_pair(const __gri
         if ((MODE & kSse) && lane == 0 && e) atomicAdd(&csse[pi], (unsigned long long)e);
     }
     __syncthreads();
+    if (MODE & kSse) init_acc_wait();
     if ((MODE & kSse) && threadIdx.x < args.nplanes && csse[threadIdx.x])
         atomicAdd(args.p[threadIdx.x].sse, csse[threadIdx.x]);
 }
@@ -428,8 +437,8 @@ inline cudaError_t launch_codec_pair(const DirectArgs& a, int num_sms, int threa
     int occ = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_codec_pair<MODE>, threads, smem);
     if (e != cudaSuccess) return e;
-    k_codec_pair<MODE><<<direct_grid(units, threads, num_sms, occ), threads, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_behind_init(k_codec_pair<MODE>, direct_grid(units, threads, num_sms, occ), threads, smem, s, a,
+                              (MODE & kSse) != 0);
 }
 
 }  // namespace dctgb
