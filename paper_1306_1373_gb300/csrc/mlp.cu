@@ -226,12 +226,15 @@ struct AdamArgs {
     float lr, b1, b2, eps, c1, c2;
 };
 
+// The fused multiply-adds are written out so that every kernel that inlines
+// this rounds alike.
+__device__ __forceinline__ void adam_step(const AdamArgs& a, float& P, float& m, float& v, float gi) {
+    m = fmaf(1.0f - a.b1, gi, __fmul_rn(a.b1, m));
+    v = fmaf(__fmul_rn(1.0f - a.b2, gi), gi, __fmul_rn(a.b2, v));
+    P = __fsub_rn(P, __fdiv_rn(__fmul_rn(a.lr, __fmul_rn(m, a.c1)), __fadd_rn(__fsqrt_rn(__fmul_rn(v, a.c2)), a.eps)));
+}
 __device__ __forceinline__ void adam_update(const AdamArgs& a, int p, float gi) {
-    const float mi = a.b1 * a.m[p] + (1.0f - a.b1) * gi;
-    const float vi = a.b2 * a.v[p] + (1.0f - a.b2) * gi * gi;
-    a.m[p] = mi;
-    a.v[p] = vi;
-    a.P[p] -= a.lr * (mi * a.c1) / (sqrtf(vi * a.c2) + a.eps);
+    adam_step(a, a.P[p], a.m[p], a.v[p], gi);
 }
 
 // ADAM: also apply the Adam step to each parameter as soon as its sum is
@@ -341,6 +344,389 @@ __global__ void k_adam(AdamArgs a, const float* __restrict__ g) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= kParams) return;
     adam_update(a, p, g[p]);
+}
+
+// ---------------------------------------------------------------------------
+// A run of training steps in one launch: one cluster of 16 CTAs
+// ---------------------------------------------------------------------------
+// A step of k_mlp_delta and k_mlp_grad is bound by latency, not by work (5.8
+// million multiply-adds): two dependent launches, the weights staged anew and
+// the cache columns fetched by few CTAs cost 24 us.  Here a cluster stays on 16
+// SMs for all steps.  Every CTA holds all weights, as 16 records of one owner's
+// four hidden units each.  Phase F: CTA c runs rows 16c..16c+15 of a group of
+// 256 through forward and deltas (a warp takes 32 units of 4 rows, so a weight
+// is loaded once for four rows).  All CTAs need all rows' inputs and first-layer
+// outputs: each CTA writes its rows to global memory and has them multicast to
+// the cluster while the rest of phase F runs (one copy per receiver instead, or
+// every CTA fetching all rows from L2, both moved about 12 bytes per clock and
+// SM: 13,000 clocks a step).  The deltas of the units a CTA owns go to it in one
+// bulk copy between shared memories.  Phase G: CTA c sums its units' gradients
+// over the rows in ascending order, applies Adam to parameters it keeps in
+// registers and multicasts its record.  Every copy is counted by the
+// receiver's mbarrier; a CTA that holds all 16 new records knows that every CTA
+// has finished its sums, so the buffers it sends into next are free, and no
+// other barrier is needed.  The inputs of the next rows load while phase G
+// runs.  All sums and updates have the operands and order of the two kernels:
+// the same bits.  16,000 rows, batch 256 (63 steps): 770 us an epoch against
+// 1540 us.
+constexpr int kCluster = 16;
+constexpr int kEpochThreads = 512;
+constexpr int kOwned = kHid / kCluster;                // hidden units a CTA owns per layer
+constexpr int kGroupRows = 256;                        // rows in flight
+constexpr int kCtaRows = kGroupRows / kCluster;
+constexpr int kEpochSteps = 64;                        // steps per launch
+// Smaller batches have no room in the workspace for the cluster's exchange
+// area, larger ones fill the GPU with the two kernels.
+constexpr int kEpochMinBatch = 64, kEpochMaxBatch = 1024;
+static_assert(kOwned == 4 && kCtaRows == 16 && kIn % 4 == 0, "phases F and G index by fours");
+
+// One owner's weights: W1 rows (80, padded to 81), W2 rows (64, padded to 65),
+// b1, b2, W3 of its four units and (owner 0) b3.  With 604 floats a record,
+// lane u reading its unit's W1 or W2 row hits bank (28 (u / 4) + 17 or 1 (u % 4))
+// mod 32: all 32 distinct.
+constexpr int kW1Row = kIn + 1, kW2Row = kHid + 1;
+constexpr int rW2 = kOwned * kW1Row, rB1 = rW2 + kOwned * kW2Row, rB2 = rB1 + 4, rW3 = rB2 + 4, rB3 = rW3 + 4,
+              kRecord = 604;
+static_assert(rB3 + 1 <= kRecord && rB1 % 4 == 0 && kRecord % 4 == 0, "record layout");
+
+struct EpochArgs {
+    float *P, *m, *v;
+    const float *feats, *labels;
+    const int* order;                 // of the first step's first row
+    const float *mean, *stdv;
+    float* loss;                      // of the first step
+    float* exch;                      // kCluster * kExch floats
+    int bf16, n, batch, nsteps;       // n rows left from the first step on
+    float lr, b1, b2, eps;
+    float c1[kEpochSteps], c2[kEpochSteps];
+};
+
+// What one CTA's 16 rows hold for one receiver: da1, da2, h2 of the
+// receiver's units and (y, dz, y - label, 0).
+struct __align__(16) Deltas {
+    float d1[kCtaRows][4], d2[kCtaRows][4], h2[kCtaRows][4], z[kCtaRows][4];
+};
+// A CTA's part of the exchange area: its rows' inputs and h1, its record.
+constexpr int xH1 = kCtaRows * kIn, xRec = xH1 + kCtaRows * kHid, kExch = xRec + kRecord;
+static_assert(kCluster * kExch <= kEpochMinBatch * kCache + 2 * kParams, "the exchange area fits the workspace");
+
+struct __align__(16) EpochSmem {
+    float w[kCluster * kRecord];               // all weights
+    float gx[kGroupRows][kIn], gh[kGroupRows][kHid];   // received: inputs and h1 of 256 rows
+    Deltas gd[kCluster];                       // received, by sender
+    float x[kCtaRows][kIn], h1[kCtaRows][kHid];        // this CTA's rows
+    Deltas sd[kCluster];                       // to send, by receiver
+    unsigned long long bar[2];                 // rows, records
+    int failed;                                // a wait ran out (the losses become NaN)
+};
+static_assert(sizeof(EpochSmem) <= 232448, "shared memory of one CTA");
+constexpr unsigned kRowBytes = (kCtaRows * (kIn + kHid)) * 4 + sizeof(Deltas);   // one CTA's rows to one receiver
+
+__device__ __forceinline__ unsigned sm_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
+}
+// Bulk copy of `bytes` from this CTA's shared memory to the same or another
+// place (dst: an address in this CTA's window) in CTA `rank`, counted on the
+// receiver's copy of mbarrier `bar`.
+__device__ __forceinline__ void send(unsigned rank, void* dst, const void* src, unsigned bytes, void* bar) {
+    unsigned d, b;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(sm_addr(dst)), "r"(rank));
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(b) : "r"(sm_addr(bar)), "r"(rank));
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(d),
+                 "r"(sm_addr(src)), "r"(bytes), "r"(b)
+                 : "memory");
+}
+// Bulk copy from global memory to `dst` in every CTA of the cluster, counted on
+// each one's mbarrier `bar`.
+__device__ __forceinline__ void multicast(void* dst, const void* src, unsigned bytes, void* bar) {
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1], %2, [%3], %4;" ::"r"(
+            sm_addr(dst)),
+        "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(sm_addr(bar)), "h"((unsigned short)0xFFFF)
+        : "memory");
+}
+// Waits for the phase of `parity` of a mbarrier, for at most about a second.
+__device__ __forceinline__ bool wait_bar(const void* bar, unsigned parity) {
+    const long long t0 = clock64();
+    unsigned ok;
+    do {
+        asm volatile("{\n\t.reg .pred p;\n\t"
+                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok)
+                     : "r"(sm_addr(bar)), "r"(parity)
+                     : "memory");
+    } while (!ok && clock64() - t0 < 2000000000ll);
+    return ok != 0;
+}
+__device__ __forceinline__ void expect_bytes(void* bar, unsigned bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;" ::"r"(sm_addr(bar)), "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
+
+// acc[r] += w x[r] over N inputs in ascending order for four rows; x(r, i)
+// gives four inputs of a row, w(i) one weight.
+template <int N, typename X, typename W>
+__device__ __forceinline__ void dot4(float (&acc)[4], X in, W w) {
+#pragma unroll 5
+    for (int i = 0; i < N; i += 4) {
+        float4 x[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) x[r] = *reinterpret_cast<const float4*>(in(r, i));
+        const float w0 = w(i), w1 = w(i + 1), w2 = w(i + 2), w3 = w(i + 3);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[r] = fmaf(w0, x[r].x, acc[r]);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[r] = fmaf(w1, x[r].y, acc[r]);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[r] = fmaf(w2, x[r].z, acc[r]);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[r] = fmaf(w3, x[r].w, acc[r]);
+    }
+}
+
+// g[u] += d(r)[u] x[r] over `rows` rows in ascending order, eight loaded ahead;
+// d(r) gives the four deltas of row r.
+template <int LD, typename D>
+__device__ __forceinline__ void grad4(float (&g)[4], const float* x, int rows, D d) {
+    int r = 0;
+    for (; r + 8 <= rows; r += 8) {
+        float xv[8];
+        float4 dv[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            xv[k] = x[(r + k) * LD];
+            dv[k] = *reinterpret_cast<const float4*>(d(r) + 4 * k);      // eight rows of one sender
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            g[0] = fmaf(dv[k].x, xv[k], g[0]);
+            g[1] = fmaf(dv[k].y, xv[k], g[1]);
+            g[2] = fmaf(dv[k].z, xv[k], g[2]);
+            g[3] = fmaf(dv[k].w, xv[k], g[3]);
+        }
+    }
+    for (; r < rows; ++r) {
+        const float4 dv = *reinterpret_cast<const float4*>(d(r));
+        g[0] = fmaf(dv.x, x[r * LD], g[0]);
+        g[1] = fmaf(dv.y, x[r * LD], g[1]);
+        g[2] = fmaf(dv.z, x[r * LD], g[2]);
+        g[3] = fmaf(dv.w, x[r * LD], g[3]);
+    }
+}
+
+__global__ void __launch_bounds__(kEpochThreads, 1) k_mlp_epoch(const __grid_constant__ EpochArgs a) {
+    extern __shared__ __align__(16) uint8_t smem_raw[];
+    EpochSmem& S = *reinterpret_cast<EpochSmem*>(smem_raw);
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int rank = blockIdx.x;                               // one cluster: CTA rank = block index
+    for (int e = t; e < kHid * kIn; e += kEpochThreads) {
+        const int u = e / kIn, i = e - u * kIn;
+        S.w[(u >> 2) * kRecord + (u & 3) * kW1Row + i] = a.P[oW1 + e];
+    }
+    for (int e = t; e < kHid * kHid; e += kEpochThreads) {
+        const int u = e / kHid, i = e - u * kHid;
+        S.w[(u >> 2) * kRecord + rW2 + (u & 3) * kW2Row + i] = a.P[oW2 + e];
+    }
+    if (t < kHid) {
+        float* r = S.w + (t >> 2) * kRecord + (t & 3);
+        r[rB1] = a.P[oB1 + t];
+        r[rB2] = a.P[oB2 + t];
+        r[rW3] = a.P[oW3 + t];
+    }
+    if (t == 0) {
+        S.w[rB3] = a.P[oB3];
+        S.failed = 0;
+        for (int k = 0; k < 2; ++k) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sm_addr(&S.bar[k])) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    float* const exch = a.exch + (size_t)rank * kExch;
+
+    // owned parameters, in registers for the whole run: threads 0..79 column t
+    // of W1 (four units), 96..159 column t - 96 of W2, the first lanes of warps
+    // 5..8 b1, b2, W3 and (CTA 0) b3, lane 0 of warp 9 the loss (each its own
+    // warp: as branches of one warp they would run one after the other)
+    int np = 0, p0 = 0, pstep = 0, rpos = 0, rstep = 0;
+    if (t < kIn) { np = 4; p0 = oW1 + kOwned * rank * kIn + t; pstep = kIn; rpos = t; rstep = kW1Row; }
+    else if (t >= 96 && t < 96 + kHid) {
+        np = 4; p0 = oW2 + kOwned * rank * kHid + t - 96; pstep = kHid; rpos = rW2 + t - 96; rstep = kW2Row;
+    } else if (warp >= 5 && warp < 8 && lane < 4) {
+        np = 1; p0 = (warp == 5 ? oB1 : warp == 6 ? oB2 : oW3) + kOwned * rank + lane; rpos = rB1 + 4 * (warp - 5) + lane;
+    } else if (warp == 8 && lane == 0 && rank == 0) { np = 1; p0 = oB3; rpos = rB3; }
+    const bool sums_loss = warp == 9 && lane == 0;
+    float P[4], M[4], V[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (u < np) {
+            P[u] = a.P[p0 + u * pstep];
+            M[u] = a.m[p0 + u * pstep];
+            V[u] = a.v[p0 + u * pstep];
+        }
+
+    // this thread's elements of the CTA's 16 x 80 inputs, loaded ahead
+    constexpr int kElems = (kCtaRows * kIn + kEpochThreads - 1) / kEpochThreads;
+    float xf[kElems], mu[kElems], sd[kElems], label = 0.0f;
+#pragma unroll
+    for (int k = 0; k < kElems; ++k) {
+        const int e = t + k * kEpochThreads;
+        mu[k] = e < kCtaRows * kIn ? a.mean[e % kIn] : 0.0f;
+        sd[k] = e < kCtaRows * kIn ? a.stdv[e % kIn] : 1.0f;
+    }
+    const int unit = 32 * (warp & 1) + lane, rq = 4 * ((warp >> 1) & 3);   // phase F, warps 0..7
+    const auto load_rows = [&](int step, int g0) {
+        const int cnt = step < a.nsteps ? min(a.batch, a.n - step * a.batch) : 0;
+        const int row0 = g0 + kCtaRows * rank;
+        const int* const index = a.order + (size_t)step * a.batch;
+#pragma unroll
+        for (int k = 0; k < kElems; ++k) {
+            const int e = t + k * kEpochThreads, r = e / kIn;
+            xf[k] = mu[k];
+            if (e < kCtaRows * kIn && row0 + r < cnt) xf[k] = __ldg(a.feats + (size_t)__ldg(index + row0 + r) * kIn + e - r * kIn);
+        }
+        const int row = row0 + rq + (lane & 3);
+        label = row < cnt ? __ldg(a.labels + __ldg(index + row)) : 0.0f;
+    };
+    load_rows(0, 0);
+    cluster_sync();                                            // mbarriers are ready everywhere
+
+    unsigned row_phase = 0;
+    for (int step = 0; step < a.nsteps; ++step) {
+        const int cnt = min(a.batch, a.n - step * a.batch);
+        float g[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        for (int g0 = 0; g0 < cnt; g0 += kGroupRows) {
+            if (g0 > 0) cluster_sync();                        // every CTA's sums over the previous rows are done
+            // ---- phase F: rows row0 .. row0 + 15 of this minibatch
+            const int row0 = g0 + kCtaRows * rank;
+            if (t == 0) expect_bytes(&S.bar[0], kCluster * kRowBytes);
+#pragma unroll
+            for (int k = 0; k < kElems; ++k) {
+                const int e = t + k * kEpochThreads;
+                if (e < kCtaRows * kIn) {
+                    const float x = (xf[k] - mu[k]) / sd[k];
+                    (&S.x[0][0])[e] = x;
+                    exch[e] = x;
+                }
+            }
+            fence_async();
+            __syncthreads();
+            if (t == 0) multicast(S.gx[kCtaRows * rank], exch, sizeof(S.x), &S.bar[0]);
+            if (warp < 8) {
+                const auto bar = [] { asm volatile("bar.sync 1, 256;" ::: "memory"); };
+                const float* const rec = S.w + (unit >> 2) * kRecord + (unit & 3);
+                const float* const w1 = S.w + (unit >> 2) * kRecord + (unit & 3) * kW1Row;
+                const float* const w2 = S.w + (unit >> 2) * kRecord + rW2 + (unit & 3) * kW2Row;
+                float a1[4], a2[4], s[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) a1[r] = rec[rB1];
+                dot4<kIn>(a1, [&](int r, int i) { return &S.x[rq + r][i]; }, [&](int i) { return w1[i]; });
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const float h = act(gelu(a1[r]), a.bf16);
+                    S.h1[rq + r][unit] = h;
+                    exch[xH1 + (rq + r) * kHid + unit] = h;
+                    a2[r] = rec[rB2];
+                }
+                fence_async();
+                bar();
+                if (t == 0) multicast(S.gh[kCtaRows * rank], exch + xH1, sizeof(S.h1), &S.bar[0]);
+                dot4<kHid>(a2, [&](int r, int i) { return &S.h1[rq + r][i]; }, [&](int i) { return w2[i]; });
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    S.sd[unit >> 2].h2[rq + r][unit & 3] = act(gelu(a2[r]), a.bf16);
+                }
+                bar();
+                // output and its delta: lane r < 4 of both warps of a row quad
+                float dz;
+                {
+                    const int r = lane & 3, row = row0 + rq + r;
+                    float z = S.w[rB3];
+#pragma unroll 8
+                    for (int j = 0; j < kHid; j += 4) {
+                        const float4 w = *reinterpret_cast<const float4*>(S.w + (j >> 2) * kRecord + rW3);
+                        const float4 h = *reinterpret_cast<const float4*>(S.sd[j >> 2].h2[rq + r]);
+                        z = fmaf(w.x, h.x, z);
+                        z = fmaf(w.y, h.y, z);
+                        z = fmaf(w.z, h.z, z);
+                        z = fmaf(w.w, h.w, z);
+                    }
+                    const float y = 1.0f / (1.0f + expf(-z));
+                    dz = row < cnt ? 2.0f * (y - label) / (float)cnt * y * (1.0f - y) : 0.0f;
+                    // every receiver's copy: 16 receivers over 8 lanes a row of two warps
+                    *reinterpret_cast<float4*>(S.sd[(lane >> 2) + 8 * (warp & 1)].z[rq + r]) =
+                        make_float4(y, dz, y - label, 0.0f);
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const float d = __shfl_sync(0xffffffffu, dz, r) * rec[rW3] * gelu_grad(a2[r]);
+                    S.sd[unit >> 2].d2[rq + r][unit & 3] = d;
+                    s[r] = 0.0f;
+                }
+                bar();
+                dot4<kHid>(s, [&](int r, int j) { return S.sd[j >> 2].d2[rq + r]; },
+                             [&](int j) { return S.w[(j >> 2) * kRecord + rW2 + (j & 3) * kW2Row + unit]; });
+#pragma unroll
+                for (int r = 0; r < 4; ++r) S.sd[unit >> 2].d1[rq + r][unit & 3] = s[r] * gelu_grad(a1[r]);
+            }
+            fence_async();
+            __syncthreads();
+            if (t < kCluster) send(t, &S.gd[rank], &S.sd[t], sizeof(Deltas), &S.bar[0]);
+            // the next rows' inputs load during phase G
+            if (g0 + kGroupRows < cnt) load_rows(step, g0 + kGroupRows);
+            else load_rows(step + 1, 0);
+
+            // ---- phase G over these rows
+            const int rows = min(kGroupRows, cnt - g0);
+            if (!S.failed && !wait_bar(&S.bar[0], row_phase & 1)) S.failed = 1;
+            ++row_phase;
+            if (t < kIn) {
+                grad4<kIn>(g, &S.gx[0][t], rows, [&](int r) { return &S.gd[r >> 4].d1[r & 15][0]; });
+            } else if (t >= 96 && t < 96 + kHid) {
+                grad4<kHid>(g, &S.gh[0][t - 96], rows, [&](int r) { return &S.gd[r >> 4].d2[r & 15][0]; });
+            } else if (warp == 5 && lane < 4) {
+#pragma unroll 16
+                for (int r = 0; r < rows; ++r) g[0] += S.gd[r >> 4].d1[r & 15][lane];
+            } else if (warp == 6 && lane < 4) {
+#pragma unroll 16
+                for (int r = 0; r < rows; ++r) g[0] += S.gd[r >> 4].d2[r & 15][lane];
+            } else if (warp == 7 && lane < 4) {
+#pragma unroll 16
+                for (int r = 0; r < rows; ++r) g[0] = fmaf(S.gd[r >> 4].z[r & 15][1], S.gd[r >> 4].h2[r & 15][lane], g[0]);
+            } else if (warp == 8 && lane == 0) {
+#pragma unroll 16
+                for (int r = 0; r < rows; ++r) g[0] += S.gd[r >> 4].z[r & 15][1];
+            } else if (sums_loss) {
+#pragma unroll 16
+                for (int r = 0; r < rows; ++r) {
+                    const float d = S.gd[r >> 4].z[r & 15][2];
+                    g[0] = fmaf(d, d, g[0]);
+                }
+            }
+        }
+        if (sums_loss && rank == 0) a.loss[step] = S.failed ? __int_as_float(0x7fc00000) : g[0] / (float)cnt;
+        if (t == 0) expect_bytes(&S.bar[1], kCluster * kRecord * 4);
+        const AdamArgs ad{nullptr, nullptr, nullptr, a.lr, a.b1, a.b2, a.eps, a.c1[step], a.c2[step]};
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (u < np) {
+                adam_step(ad, P[u], M[u], V[u], g[u]);
+                exch[xRec + rpos + u * rstep] = P[u];
+            }
+        fence_async();
+        __syncthreads();
+        if (t == 0) multicast(S.w + kRecord * rank, exch + xRec, kRecord * 4, &S.bar[1]);
+        if (!S.failed && !wait_bar(&S.bar[1], step & 1)) S.failed = 1;
+        __syncthreads();
+    }
+    cluster_sync();                                            // no CTA leaves while another still sends to it
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (u < np) {
+            a.P[p0 + u * pstep] = P[u];
+            a.m[p0 + u * pstep] = M[u];
+            a.v[p0 + u * pstep] = V[u];
+        }
 }
 
 // training target of a quality label: (Q - 1) / 99 (IEEE division, as the
@@ -454,6 +840,30 @@ static cudaError_t launch_train_step(const dct_mlp* net, const float* feats, con
     return cudaGetLastError();
 }
 
+// Whether this device can hold the training cluster (16 CTAs of one cluster
+// need one GPC with as many SMs free of other limits).
+static bool epoch_cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, cudaStream_t s) {
+    cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3(kCluster);
+    cfg.blockDim = dim3(kEpochThreads);
+    cfg.dynamicSmemBytes = sizeof(EpochSmem);
+    cfg.stream = s;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kCluster;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaFuncSetAttribute(k_mlp_epoch, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaFuncSetAttribute(k_mlp_epoch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(EpochSmem)) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&clusters, k_mlp_epoch, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return clusters >= 1;
+}
+
 static dct_status check_net(const dct_mlp* net, bool train) {
     if (!net || !net->params || !net->feat_mean || !net->feat_std)
         return fail(DCT_ERR_INVALID_ARG, "network pointers are null");
@@ -541,9 +951,46 @@ dct_status dct_mlp_train_epoch(dct_mlp* net, const float* feats, const float* la
     if (n < 1 || batch < 1 || batch > (1 << 20)) return fail(DCT_ERR_INVALID_ARG, "n >= 1 and batch in 1..2^20");
     if (!adam_params_ok(lr, 0.9f, 0.999f, 1e-8f)) return fail(DCT_ERR_INVALID_ARG, "learning rate must be > 0");
     if (((uintptr_t)workspace) & 15u) return fail(DCT_ERR_INVALID_ARG, "workspace must be 16-byte aligned");
-    float* grad = reinterpret_cast<float*>(static_cast<char*>(workspace) + dct_mlp_workspace_bytes(batch));
+    // batches that one cluster handles: runs of steps in one launch
+    cudaStream_t st_ = (cudaStream_t)stream;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at;
+    if (batch >= kEpochMinBatch && batch <= kEpochMaxBatch && epoch_cluster_config(cfg, at, st_)) {
+        const int steps = (n + batch - 1) / batch;
+        for (int k0 = 0; k0 < steps; k0 += kEpochSteps) {
+            EpochArgs a;
+            memset(&a, 0, sizeof a);
+            a.nsteps = steps - k0 < kEpochSteps ? steps - k0 : kEpochSteps;
+            for (int k = 0; k < a.nsteps; ++k) {
+                const AdamArgs s = next_adam_step(net, lr, 0.9f, 0.999f, 1e-8f);
+                a.c1[k] = s.c1;
+                a.c2[k] = s.c2;
+                a.b1 = s.b1;
+                a.b2 = s.b2;
+                a.eps = s.eps;
+            }
+            a.lr = lr;
+            a.P = net->params;
+            a.m = net->adam_m;
+            a.v = net->adam_v;
+            a.feats = feats;
+            a.labels = labels;
+            a.order = order + (size_t)k0 * batch;
+            a.mean = net->feat_mean;
+            a.stdv = net->feat_std;
+            a.loss = loss_out + k0;
+            a.exch = static_cast<float*>(workspace);
+            a.bf16 = net->act_bf16;
+            a.n = n - k0 * batch;
+            a.batch = batch;
+            cudaError_t e = cudaLaunchKernelEx(&cfg, k_mlp_epoch, a);
+            if (e != cudaSuccess) return cuda_fail(e, "training launch");
+        }
+        return DCT_OK;
+    }
     // per minibatch: the delta kernel, then the gradient sums with the Adam
     // step fused (same arithmetic as dct_mlp_loss_grad + dct_mlp_adam)
+    float* grad = reinterpret_cast<float*>(static_cast<char*>(workspace) + dct_mlp_workspace_bytes(batch));
     for (int b0 = 0, k = 0; b0 < n; b0 += batch, ++k) {
         const int cnt = n - b0 < batch ? n - b0 : batch;
         cudaError_t e = launch_train_step<true>(net, feats, labels, order + b0, cnt, grad, loss_out + k, workspace,
