@@ -540,27 +540,37 @@ __device__ __forceinline__ unsigned process_tile(const PlaneArg& P, const QuantS
         }
 
         if (MODE & kStats) {
-            unsigned s = 0, s2 = 0, mn = 255, mx = 0, adx = 0, ady = 0, dx2 = 0, dy2 = 0;
+            // four samples at a time: byte dot products, absolute
+            // differences, minima and maxima (2.8 instructions per sample
+            // against 14 one by one)
+            unsigned s = 0, s2 = 0, adx = 0, ady = 0, dx2 = 0, dy2 = 0;
+            unsigned mn4 = 0xFFFFFFFFu, mx4 = 0u;
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
+                // right neighbours; the last column's is itself
+                const uint32_t right[2] = {__funnelshift_r(pix[r][0], pix[r][1], 8), __byte_perm(pix[r][1], 0, 0x3321)};
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const int p = sample(pix, r, c);
-                    s += p;
-                    s2 += p * p;
-                    mn = min(mn, (unsigned)p);
-                    mx = max(mx, (unsigned)p);
-                    if (c < 7) {
-                        const int d = sample(pix, r, c + 1) - p;
-                        adx += abs(d);
-                        dx2 += d * d;
-                    }
+                for (int h = 0; h < 2; ++h) {
+                    const uint32_t p = pix[r][h];
+                    s = __dp4a(p, 0x01010101u, s);
+                    s2 = __dp4a(p, p, s2);
+                    mn4 = __vminu4(mn4, p);
+                    mx4 = __vmaxu4(mx4, p);
+                    const uint32_t dx = __vabsdiffu4(p, right[h]);
+                    adx = __dp4a(dx, 0x01010101u, adx);
+                    dx2 = __dp4a(dx, dx, dx2);
                     if (r < 7) {
-                        const int d = sample(pix, r + 1, c) - p;
-                        ady += abs(d);
-                        dy2 += d * d;
+                        const uint32_t dy = __vabsdiffu4(p, pix[r + 1][h]);
+                        ady = __dp4a(dy, 0x01010101u, ady);
+                        dy2 = __dp4a(dy, dy, dy2);
                     }
                 }
+            }
+            unsigned mn = 255, mx = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                mn = min(mn, (mn4 >> (8 * k)) & 0xFFu);
+                mx = max(mx, (mx4 >> (8 * k)) & 0xFFu);
             }
             if (!active) { s = s2 = adx = ady = dx2 = dy2 = 0; mn = 255; mx = 0; }
             const unsigned vals[8] = {warp_sum(s), warp_sum(s2), __reduce_min_sync(0xffffffffu, mn),

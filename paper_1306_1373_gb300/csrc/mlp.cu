@@ -1,10 +1,12 @@
 // Learned rate controller, network side: the 80 features, input
 // normalisation, forward pass, back-propagation with deterministic
 // (fixed-order) minibatch sums, and Adam.  The network is tiny (9409
-// parameters), so it runs on plain FMA units: one thread per sample for
-// inference, one warp per minibatch row for the training forward and delta
-// pass, one thread per parameter for the gradient sums (in tiles that stage
-// the minibatch in shared memory) and the update.
+// parameters), so it runs on plain FMA units: one warp per sample for
+// inference, one cluster of 16 CTAs for a run of training steps; single
+// gradients and the smallest and largest batches use one warp per minibatch
+// row for the forward and delta pass and one thread per parameter for the
+// gradient sums (in tiles that stage the minibatch in shared memory) and the
+// update.
 #include <cmath>
 #include <cstring>
 
@@ -34,69 +36,81 @@ __device__ __forceinline__ float act(float h, int bf16) {
     return bf16 ? __bfloat162float(__float2bfloat16_rn(h)) : h;
 }
 
-// Forward pass of one sample; fills the cache when c != nullptr.
-__device__ float forward_sample(const float* __restrict__ P, const float* __restrict__ x,
-                                const float* __restrict__ mean, const float* __restrict__ stdv, int bf16,
-                                float* __restrict__ c) {
-    float xn[kIn];
-#pragma unroll
-    for (int i = 0; i < kIn; ++i) {
-        xn[i] = (x[i] - mean[i]) / stdv[i];
-        if (c) c[cXn + i] = xn[i];
-    }
-    float h1[kHid];
-    for (int j = 0; j < kHid; ++j) {
-        float a = P[oB1 + j];
-        const float* w = P + oW1 + j * kIn;
-#pragma unroll
-        for (int i = 0; i < kIn; ++i) a = fmaf(w[i], xn[i], a);
-        h1[j] = act(gelu(a), bf16);
-        if (c) {
-            c[cA1 + j] = a;
-            c[cH1 + j] = h1[j];
-        }
-    }
-    float z = P[oB3];
-    for (int j = 0; j < kHid; ++j) {
-        float a = P[oB2 + j];
-        const float* w = P + oW2 + j * kHid;
-#pragma unroll
-        for (int i = 0; i < kHid; ++i) a = fmaf(w[i], h1[i], a);
-        const float h = act(gelu(a), bf16);
-        if (c) {
-            c[cA2 + j] = a;
-            c[cH2 + j] = h;
-        }
-        z = fmaf(P[oW3 + j], h, z);
-    }
-    const float y = 1.0f / (1.0f + expf(-z));
-    if (c) c[cY] = y;
-    return y;
-}
+// Inference, one warp per sample: lane l owns hidden units l and l + 32 of both
+// layers, every sum over its inputs in ascending order (the inputs a lane does
+// not hold come by shuffle).  W1 and W2 are staged transposed with rows padded
+// to 65 floats, as in k_mlp_delta.  One thread per sample took 219 us for the
+// 48 frames of a small rate-control call (a serial walk over 9,409 parameters
+// in global memory); this takes 10 us.
+constexpr int kFwdRows = 8;                    // samples (warps) per CTA
+constexpr int kTStride = kHid + 1;             // padded row of a transposed weight matrix
 
-__global__ void k_mlp_forward(const float* __restrict__ P, const float* __restrict__ feats,
-                              const float* __restrict__ mean, const float* __restrict__ stdv, int bf16, int n,
-                              float* __restrict__ y_out, int* __restrict__ q_out) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    const float y = forward_sample(P, feats + (size_t)s * kIn, mean, stdv, bf16, nullptr);
-    if (y_out) y_out[s] = y;
-    if (q_out) {
-        const float q = rintf(1.0f + 99.0f * y);
-        q_out[s] = (int)fminf(100.0f, fmaxf(1.0f, q));
+__global__ void __launch_bounds__(kFwdRows * 32)
+k_mlp_forward(const float* __restrict__ P, const float* __restrict__ feats, const float* __restrict__ mean,
+              const float* __restrict__ stdv, int bf16, int n, float* __restrict__ y_out, int* __restrict__ q_out) {
+    __shared__ float w1t[kIn * kTStride];       // w1t[i * 65 + j] = W1[j][i]
+    __shared__ float w2t[kHid * kTStride];
+#pragma unroll 8
+    for (int e = threadIdx.x; e < kHid * kIn; e += kFwdRows * 32) w1t[(e % kIn) * kTStride + e / kIn] = P[oW1 + e];
+#pragma unroll 8
+    for (int e = threadIdx.x; e < kHid * kHid; e += kFwdRows * 32) w2t[(e % kHid) * kTStride + e / kHid] = P[oW2 + e];
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int s = blockIdx.x * kFwdRows + (threadIdx.x >> 5); s < n; s += gridDim.x * kFwdRows) {   // warp-uniform
+        const float* x = feats + (size_t)s * kIn;
+        float xn[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int i = lane + 32 * k;
+            xn[k] = i < kIn ? (x[i] - mean[i]) / stdv[i] : 0.0f;
+        }
+        float a[2], h[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) a[k] = P[oB1 + lane + 32 * k];
+#pragma unroll
+        for (int i = 0; i < kIn; ++i) {
+            const float v = __shfl_sync(0xffffffffu, xn[i >> 5], i & 31);
+#pragma unroll
+            for (int k = 0; k < 2; ++k) a[k] = fmaf(w1t[i * kTStride + lane + 32 * k], v, a[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            h[k] = act(gelu(a[k]), bf16);
+            a[k] = P[oB2 + lane + 32 * k];
+        }
+#pragma unroll
+        for (int i = 0; i < kHid; ++i) {
+            const float v = __shfl_sync(0xffffffffu, h[i >> 5], i & 31);
+#pragma unroll
+            for (int k = 0; k < 2; ++k) a[k] = fmaf(w2t[i * kTStride + lane + 32 * k], v, a[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) h[k] = act(gelu(a[k]), bf16);
+        const float w3[2] = {P[oW3 + lane], P[oW3 + lane + 32]};
+        float z = P[oB3];
+#pragma unroll
+        for (int j = 0; j < kHid; ++j)
+            z = fmaf(__shfl_sync(0xffffffffu, w3[j >> 5], j & 31), __shfl_sync(0xffffffffu, h[j >> 5], j & 31), z);
+        const float y = 1.0f / (1.0f + expf(-z));
+        if (lane == 0) {
+            if (y_out) y_out[s] = y;
+            if (q_out) {
+                const float q = rintf(1.0f + 99.0f * y);
+                q_out[s] = (int)fminf(100.0f, fmaxf(1.0f, q));
+            }
+        }
     }
 }
 
 // forward + output delta + hidden deltas of one minibatch row per warp:
 // lane l owns hidden units l and l + 32 of both layers; every sum runs over
-// its inputs in ascending order as forward_sample's does (the inputs a lane
+// its inputs in ascending order as k_mlp_forward's does (the inputs a lane
 // does not hold come by shuffle), so the cache holds the same values.  The
 // CTA first stages W1 and W2 transposed in shared memory with rows padded
 // to 65 floats: the forward sums read W^T[i][lane] and the backward sum
 // reads W2[j][lane] = W2^T[lane][j], both free of bank conflicts (reading
 // W1 straight from global memory touched 32 cache lines per warp access).
 constexpr int kDeltaRows = 8;                  // minibatch rows (warps) per CTA
-constexpr int kTStride = kHid + 1;             // padded row of a transposed weight matrix
 
 __global__ void __launch_bounds__(kDeltaRows * 32)
 k_mlp_delta(const float* __restrict__ P, const float* __restrict__ feats, const float* __restrict__ labels,
@@ -773,43 +787,52 @@ k_feat_norm(const float* __restrict__ feats, int n, float* __restrict__ mean, fl
     }
 }
 
-// the 80 features of one frame from its statistics words (float64 arithmetic)
+// Feature k of one frame from its statistics words (float64 arithmetic), one
+// thread each: one thread per frame took 104 us for 48 frames, nearly all of
+// it the 64 logarithms one after the other.
 __global__ void k_features(const unsigned long long* __restrict__ stats, const int* __restrict__ width,
                            const int* __restrict__ height, const float* __restrict__ target, int n,
                            float* __restrict__ out) {
-    const int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f >= n) return;
+    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= (long long)n * kIn) return;
+    const int f = (int)(e / kIn), k = (int)(e - (long long)f * kIn);
     const unsigned long long* st = stats + (size_t)f * kStatsWords;
-    float* o = out + (size_t)f * kIn;
-    const double nb = (double)st[kStBlocks], ns = (double)st[kStSamples];
-    for (int k = 0; k < 64; ++k) o[k] = (float)log1p((double)st[k] / nb);
-    const double mean = (double)st[kStSum] / ns;
-    double var = (double)st[kStSum2] / ns - mean * mean;
-    if (var < 0.0) var = 0.0;
-    o[64] = (float)(mean / 128.0);
-    o[65] = (float)(sqrt(var) / 64.0);
-    o[66] = (float)((double)st[kStMin] / 255.0);
-    o[67] = (float)((double)st[kStMax] / 255.0);
-    const double nd = nb * 56.0;
-    o[68] = (float)((double)st[kStAbsDx] / nd / 32.0);
-    o[69] = (float)((double)st[kStAbsDy] / nd / 32.0);
-    o[70] = (float)(sqrt((double)st[kStDx2] / nd) / 32.0);
-    o[71] = (float)(sqrt((double)st[kStDy2] / nd) / 32.0);
-    for (int k = 0; k < 4; ++k) o[72 + k] = (float)((double)st[kStLowAc + k] / nb);
-    o[76] = (float)(log2((double)width[f]) / 11.0);
-    o[77] = (float)(log2((double)height[f]) / 11.0);
-    o[78] = (float)(((double)target[f] - 35.0) / 7.0);
-    o[79] = 1.0f;
+    const double nb = (double)st[kStBlocks], ns = (double)st[kStSamples], nd = nb * 56.0;
+    float o = 1.0f;
+    if (k < 64) {
+        o = (float)log1p((double)st[k] / nb);
+    } else if (k == 64) {
+        o = (float)((double)st[kStSum] / ns / 128.0);
+    } else if (k == 65) {
+        const double mean = (double)st[kStSum] / ns;
+        double var = (double)st[kStSum2] / ns - mean * mean;
+        if (var < 0.0) var = 0.0;
+        o = (float)(sqrt(var) / 64.0);
+    } else if (k == 66 || k == 67) {
+        o = (float)((double)st[k == 66 ? kStMin : kStMax] / 255.0);
+    } else if (k == 68 || k == 69) {
+        o = (float)((double)st[k == 68 ? kStAbsDx : kStAbsDy] / nd / 32.0);
+    } else if (k == 70 || k == 71) {
+        o = (float)(sqrt((double)st[k == 70 ? kStDx2 : kStDy2] / nd) / 32.0);
+    } else if (k < 76) {
+        o = (float)((double)st[kStLowAc + k - 72] / nb);
+    } else if (k == 76 || k == 77) {
+        o = (float)(log2((double)(k == 76 ? width : height)[f]) / 11.0);
+    } else if (k == 78) {
+        o = (float)(((double)target[f] - 35.0) / 7.0);
+    }
+    out[e] = o;
 }
 
 cudaError_t launch_features(const unsigned long long* stats, const int* w, const int* h, const float* t, int n,
                             float* out, cudaStream_t s) {
-    k_features<<<(n + 127) / 128, 128, 0, s>>>(stats, w, h, t, n, out);
+    k_features<<<(unsigned)(((long long)n * kIn + 127) / 128), 128, 0, s>>>(stats, w, h, t, n, out);
     return cudaGetLastError();
 }
 
 cudaError_t launch_mlp_forward(const dct_mlp* net, const float* feats, int n, float* y, int* q, cudaStream_t s) {
-    k_mlp_forward<<<(n + 63) / 64, 64, 0, s>>>(net->params, feats, net->feat_mean, net->feat_std, net->act_bf16, n,
+    const int ctas = (n + kFwdRows - 1) / kFwdRows;
+    k_mlp_forward<<<ctas < 1024 ? ctas : 1024, kFwdRows * 32, 0, s>>>(net->params, feats, net->feat_mean, net->feat_std, net->act_bf16, n,
                                                y, q);
     return cudaGetLastError();
 }

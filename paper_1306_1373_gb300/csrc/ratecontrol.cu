@@ -53,7 +53,6 @@ struct RcState {
     int32_t* d_mid = nullptr;
     int32_t* d_rej = nullptr;     // last rejected quality (0: none) and its SSE
     unsigned long long* d_rej_sse = nullptr;
-    unsigned long long* d_fsse = nullptr;
     unsigned int* d_counter = nullptr;   // tile counter of the SSE passes
     // pinned host staging
     unsigned long long* h_thr = nullptr;
@@ -73,69 +72,75 @@ struct RcState {
 // table index of every plane of a slot frame for that frame's quality; clears
 // the planes' SSE words and the next pass's tile counter
 __global__ void k_rc_set_quality(PlaneArg* items, int nitems, int k, const int32_t* __restrict__ frame,
-                                 const int32_t* __restrict__ q_slot, const int32_t* __restrict__ q_global,
-                                 unsigned int* tile_counter) {
+                                 const int32_t* __restrict__ q_global, unsigned int* tile_counter) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) *tile_counter = 0u;
     if (i >= nitems) return;
     const int f = i / k;
-    const int q = q_slot ? q_slot[f] : q_global[frame[f]];
+    const int q = q_global[frame[f]];
     items[i].table = (i % k ? 100 : 0) + q - 1;
     *items[i].sse = 0ull;
 }
 
-__global__ void k_rc_frame_sse(const PlaneArg* __restrict__ items, int nframes, int k,
-                               unsigned long long* __restrict__ fsse) {
-    const int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f >= nframes) return;
+// SSE of a slot frame: the sum over its planes
+__device__ __forceinline__ unsigned long long frame_sse(const PlaneArg* __restrict__ items, int f, int k) {
     unsigned long long s = 0ull;
     for (int p = 0; p < k; ++p) s += *items[f * k + p].sse;
-    fsse[f] = s;
+    return s;
 }
 
 // learned path: keep the prediction when its SSE lies in the 0.25 dB band
-__global__ void k_rc_decide(const unsigned long long* __restrict__ fsse, const unsigned long long* __restrict__ blo,
+__global__ void k_rc_decide(const PlaneArg* __restrict__ items, int k, const unsigned long long* __restrict__ blo,
                             const unsigned long long* __restrict__ bhi, int n, unsigned long long* __restrict__ sse,
                             uint8_t* __restrict__ fell) {
     const int f = blockIdx.x * blockDim.x + threadIdx.x;
     if (f >= n) return;
-    const unsigned long long s = fsse[f];
+    const unsigned long long s = frame_sse(items, f, k);
     sse[f] = s;
     fell[f] = (s >= blo[f] && s <= bhi[f]) ? 0 : 1;
 }
 
-__global__ void k_bisect_init(int32_t* lo, int32_t* hi, int32_t* rej, int n) {
+// Everything between two passes of the bisection in one launch: takes the
+// SSEs of the pass before (except ahead of the first), narrows each slot
+// frame's interval, and sets up its planes for the next quality: their table
+// index, their cleared SSE words and the tile counter.  (Four launches of this
+// size a step took 10 us between passes, this one 3.)
+__global__ void k_bisect_step(PlaneArg* items, int n, int k, const int32_t* __restrict__ frame,
+                              const unsigned long long* __restrict__ thr, int32_t* lo, int32_t* hi, int32_t* mid,
+                              int32_t* rej, unsigned long long* rej_sse, int first, unsigned int* tile_counter) {
     const int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f < n) {
-        lo[f] = 1;
-        hi[f] = 100;
-        rej[f] = 0;
-    }
-}
-
-__global__ void k_bisect_mid(const int32_t* __restrict__ lo, const int32_t* __restrict__ hi, int32_t* mid, int n) {
-    const int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f < n) mid[f] = min(100, (lo[f] + hi[f]) >> 1);
-}
-
-__global__ void k_bisect_update(const unsigned long long* __restrict__ fsse, const int32_t* __restrict__ frame,
-                                const unsigned long long* __restrict__ thr, const int32_t* __restrict__ mid,
-                                int32_t* lo, int32_t* hi, int32_t* rej, unsigned long long* rej_sse, int n) {
-    const int f = blockIdx.x * blockDim.x + threadIdx.x;
+    if (f == 0) *tile_counter = 0u;
     if (f >= n) return;
-    if (fsse[f] <= thr[frame[f]]) {
-        hi[f] = mid[f];
+    int l = 1, h = 100;
+    if (first) {
+        rej[f] = 0;
     } else {
-        lo[f] = mid[f] + 1;
-        rej[f] = mid[f];
-        rej_sse[f] = fsse[f];
+        const unsigned long long s = frame_sse(items, f, k);
+        const int m = mid[f];
+        l = lo[f];
+        h = hi[f];
+        if (s <= thr[frame[f]]) {
+            h = m;
+        } else {
+            l = m + 1;
+            rej[f] = m;
+            rej_sse[f] = s;
+        }
+    }
+    lo[f] = l;
+    hi[f] = h;
+    const int q = min(100, (l + h) >> 1);
+    mid[f] = q;
+    for (int p = 0; p < k; ++p) {
+        items[f * k + p].table = (p ? 100 : 0) + q - 1;
+        *items[f * k + p].sse = 0ull;
     }
 }
 
 // Results to the global arrays.  The last step's mid is Q*; when its PSNR
 // lies outside the +-0.25 dB band but the last rejected quality (Q* - 1
 // whenever a step rejected) lies inside it, that quality is the result.
-__global__ void k_bisect_finish(const unsigned long long* __restrict__ fsse, const int32_t* __restrict__ frame,
+__global__ void k_bisect_finish(const PlaneArg* __restrict__ items, int k, const int32_t* __restrict__ frame,
                                 const int32_t* __restrict__ mid, const int32_t* __restrict__ rej,
                                 const unsigned long long* __restrict__ rej_sse, const unsigned long long* __restrict__ blo,
                                 const unsigned long long* __restrict__ bhi, int n, int32_t* q, unsigned long long* sse) {
@@ -143,7 +148,7 @@ __global__ void k_bisect_finish(const unsigned long long* __restrict__ fsse, con
     if (f >= n) return;
     const int g = frame[f];
     int qq = mid[f];
-    unsigned long long s = fsse[f];
+    unsigned long long s = frame_sse(items, f, k);
     const bool in_band = s >= blo[g] && s <= bhi[g];
     if (!in_band && rej[f] > 0 && rej_sse[f] >= blo[g] && rej_sse[f] <= bhi[g]) {
         qq = rej[f];
@@ -181,7 +186,7 @@ static void release_rc(RcState* r) {
     free_list(r->sub);
     void* dev[] = {r->d_item_sse, r->d_stats, r->d_feats, r->d_target, r->d_w, r->d_h, r->d_q, r->d_sse,
                    r->d_fell, r->d_thr, r->d_blo, r->d_bhi, r->d_lo, r->d_hi, r->d_mid, r->d_rej, r->d_rej_sse,
-                   r->d_fsse, r->d_counter};
+                   r->d_counter};
     for (void* p : dev) cudaFree(p);
     void* host[] = {r->h_thr, r->h_blo, r->h_bhi, r->h_target, r->h_w, r->h_h, r->h_fell};
     for (void* p : host) cudaFreeHost(p);
@@ -235,7 +240,6 @@ static dct_status ensure_rc(dct_plan_t plan, cudaStream_t s) {
     if (e == cudaSuccess) e = dalloc(&r->d_mid, cap);
     if (e == cudaSuccess) e = dalloc(&r->d_rej, cap);
     if (e == cudaSuccess) e = dalloc(&r->d_rej_sse, cap);
-    if (e == cudaSuccess) e = dalloc(&r->d_fsse, cap);
     if (e == cudaSuccess) e = dalloc(&r->d_counter, 1);
     if (e == cudaSuccess) e = halloc(&r->h_thr, cap);
     if (e == cudaSuccess) e = halloc(&r->h_blo, cap);
@@ -304,21 +308,15 @@ static inline int blocks_for(int n) { return (n + 127) / 128; }
 // 8-step bisection over the frames of list w; results to d_q / d_sse.
 static dct_status run_bisection(dct_plan_t plan, RcState* r, WorkList& w, int k, cudaStream_t s) {
     const int n = w.nframes;
-    k_bisect_init<<<blocks_for(n), 128, 0, s>>>(r->d_lo, r->d_hi, r->d_rej, n);
     for (int step = 0; step < kBisectSteps; ++step) {
-        k_bisect_mid<<<blocks_for(n), 128, 0, s>>>(r->d_lo, r->d_hi, r->d_mid, n);
-        k_rc_set_quality<<<blocks_for(w.nitems), 128, 0, s>>>(w.d_items, w.nitems, k, w.d_frame, r->d_mid, nullptr,
-                                                              r->d_counter);
+        k_bisect_step<<<blocks_for(n), 128, 0, s>>>(w.d_items, n, k, w.d_frame, r->d_thr, r->d_lo, r->d_hi, r->d_mid,
+                                                    r->d_rej, r->d_rej_sse, step == 0, r->d_counter);
         cudaError_t e = batch_launch(kLoadPix | kInverse | kSse, w.d_items, w.d_tb, r->d_bank, w.nitems, w.ntiles,
                                      plan, s, r->d_counter);
         if (e != cudaSuccess) return cuda_fail(e, "bisection pass");
-        k_rc_frame_sse<<<blocks_for(n), 128, 0, s>>>(w.d_items, n, k, r->d_fsse);
-        if (step + 1 < kBisectSteps)
-            k_bisect_update<<<blocks_for(n), 128, 0, s>>>(r->d_fsse, w.d_frame, r->d_thr, r->d_mid, r->d_lo, r->d_hi,
-                                                          r->d_rej, r->d_rej_sse, n);
     }
     // after 7 steps lo == hi on 1..100, so the 8th step evaluated Q*
-    k_bisect_finish<<<blocks_for(n), 128, 0, s>>>(r->d_fsse, w.d_frame, r->d_mid, r->d_rej, r->d_rej_sse, r->d_blo,
+    k_bisect_finish<<<blocks_for(n), 128, 0, s>>>(w.d_items, k, w.d_frame, r->d_mid, r->d_rej, r->d_rej_sse, r->d_blo,
                                                   r->d_bhi, n, r->d_q, r->d_sse);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? DCT_OK : cuda_fail(e, "bisection launch");
@@ -437,12 +435,11 @@ dct_status dct_rate_control(dct_plan_t plan, const dct_plane* planes, int planes
             return cuda_fail(e, "network launch");
         if ((st = build_list(r, r->all, planes, k, all, false, s)) != DCT_OK) return st;
         k_rc_set_quality<<<blocks_for(r->all.nitems), 128, 0, s>>>(r->all.d_items, r->all.nitems, k, r->all.d_frame,
-                                                                   nullptr, r->d_q, r->d_counter);
+                                                                   r->d_q, r->d_counter);
         e = batch_launch(kLoadPix | kInverse | kSse, r->all.d_items, r->all.d_tb, r->d_bank, r->all.nitems,
                          r->all.ntiles, plan, s, r->d_counter);
         if (e != cudaSuccess) return cuda_fail(e, "verification pass");
-        k_rc_frame_sse<<<blocks_for(nframes), 128, 0, s>>>(r->all.d_items, nframes, k, r->d_fsse);
-        k_rc_decide<<<blocks_for(nframes), 128, 0, s>>>(r->d_fsse, r->d_blo, r->d_bhi, nframes, r->d_sse, r->d_fell);
+        k_rc_decide<<<blocks_for(nframes), 128, 0, s>>>(r->all.d_items, k, r->d_blo, r->d_bhi, nframes, r->d_sse, r->d_fell);
         passes += nframes;
         e = cudaMemcpyAsync(r->h_fell, r->d_fell, nframes, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
