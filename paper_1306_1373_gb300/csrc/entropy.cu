@@ -201,9 +201,8 @@ extern "C" dct_status dct_entropy_stats(dct_plan_t plan, const int16_t* coeffs, 
     cudaError_t e = cudaMemsetAsync(stats_out, 0, sizeof(uint64_t) * kEntWords * nplanes, s);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
     int occ = 0;
-    e = cudaFuncSetAttribute(k_entropy, cudaFuncAttributeMaxDynamicSharedMemorySize, kEntSmem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_entropy, kEntThreads, kEntSmem);
-    if (e != cudaSuccess) return cuda_fail(e, "entropy kernel attributes");
+    static OccCache cache;
+    if ((e = kernel_occupancy(k_entropy, cache, kEntThreads, kEntSmem, kEntSmem, occ)) != cudaSuccess) return cuda_fail(e, "entropy kernel attributes");
     k_entropy<<<direct_grid(tiles, kEntThreads, plan->num_sms, occ), kEntThreads, kEntSmem, s>>>(a);
     e = cudaGetLastError();
     return e == cudaSuccess ? DCT_OK : cuda_fail(e, "entropy launch");

@@ -272,11 +272,8 @@ __global__ void __launch_bounds__(kExactThreads, 6) k_exact(const __grid_constan
 template <bool STORE_COEF, bool STORE_RECON>
 static cudaError_t launch_exact(const ExactArgs& a, int num_sms, cudaStream_t s) {
     int occ = 0;
-    cudaError_t e = cudaFuncSetAttribute(k_exact<STORE_COEF, STORE_RECON>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kExactSmem);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_exact<STORE_COEF, STORE_RECON>, kExactThreads,
-                                                          kExactSmem);
+    static OccCache cache;
+    cudaError_t e = kernel_occupancy(k_exact<STORE_COEF, STORE_RECON>, cache, kExactThreads, kExactSmem, kExactSmem, occ);
     if (e != cudaSuccess) return e;
     k_exact<STORE_COEF, STORE_RECON>
         <<<direct_grid(2 * a.ntiles, kExactThreads, num_sms, occ), kExactThreads, kExactSmem, s>>>(a);

@@ -9,10 +9,9 @@ template <unsigned MODE>
 static cudaError_t launch_mode(const DirectArgs& a, int num_sms, int threads, cudaStream_t s) {
     while (threads > 64 && (long long)a.ntiles < (long long)num_sms * (threads / 32)) threads /= 2;
     const size_t smem = codec_smem_bytes(threads);
-    cudaError_t e = cudaFuncSetAttribute(k_codec<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    static OccCache cache;
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_codec<MODE>, threads, smem);
+    cudaError_t e = kernel_occupancy(k_codec<MODE>, cache, threads, smem, codec_smem_bytes(kDirectThreads), occ);
     if (e != cudaSuccess) return e;
     return launch_behind_init(k_codec<MODE>, direct_grid(a.ntiles, threads, num_sms, occ), threads, smem, s, a,
                               (MODE & kStats) != 0);

@@ -432,10 +432,9 @@ inline cudaError_t launch_codec_pair(const DirectArgs& a, int num_sms, int threa
     const int units = 2 * a.ntiles;
     while (threads > 64 && (long long)units < (long long)num_sms * (threads / 32)) threads /= 2;
     const size_t smem = pair_codec_smem_bytes(threads);
-    cudaError_t e = cudaFuncSetAttribute(k_codec_pair<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    static OccCache cache;
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_codec_pair<MODE>, threads, smem);
+    cudaError_t e = kernel_occupancy(k_codec_pair<MODE>, cache, threads, smem, pair_codec_smem_bytes(kDirectThreads), occ);
     if (e != cudaSuccess) return e;
     return launch_behind_init(k_codec_pair<MODE>, direct_grid(units, threads, num_sms, occ), threads, smem, s, a,
                               (MODE & kSse) != 0);

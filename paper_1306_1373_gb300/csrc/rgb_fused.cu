@@ -232,10 +232,9 @@ extern "C" dct_status dct_compress_rgb(dct_plan_t plan, const uint8_t* rgb, int3
     a.cb_offset = (int64_t)a.nbx_y * a.nby_y * 64;
     a.cr_offset = a.cb_offset + (int64_t)a.nbx_c * a.nby_c * 64;
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = cudaFuncSetAttribute(k_compress_rgb, cudaFuncAttributeMaxDynamicSharedMemorySize, kRgbSmem);
+    static OccCache cache;
     int occ = 0;
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_compress_rgb, kRgbThreads, kRgbSmem);
+    cudaError_t e = kernel_occupancy(k_compress_rgb, cache, kRgbThreads, kRgbSmem, kRgbSmem, occ);
     if (e != cudaSuccess) return cuda_fail(e, "rgb kernel attributes");
     const int64_t cap = (int64_t)plan->num_sms * (occ > 0 ? occ : 1);
     const int grid = (int)(units < cap ? units : cap);

@@ -186,9 +186,14 @@ def _check(status, lib=None):
 
 
 def _stream_ptr(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    """Address of the given stream, or of torch's current one.  The raw query
+    costs 0.2 us of host time, torch.cuda.current_stream() 3 us of the 12.5 us
+    that a small direct call took."""
+    if stream is not None:
+        return stream.cuda_stream
+    if not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _require_cuda(*tensors):
