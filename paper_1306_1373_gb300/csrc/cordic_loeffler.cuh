@@ -1,5 +1,6 @@
 // Device flow graphs of the Cordic-based Loeffler 8-point DCT (Sec. 2.5.2,
-// Fig. 1) and its transpose, in int32 registers.
+// Fig. 1) and its transpose: the forward graph on exact integers in float32,
+// the inverse in int32 registers.
 //
 // Forward graph (standard Loeffler structure, four stages in series):
 //   stage 1  s_n = x_n + x_{7-n}, d_n = x_n - x_{7-n}
