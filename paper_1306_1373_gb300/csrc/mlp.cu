@@ -611,6 +611,7 @@ __global__ void __launch_bounds__(kEpochThreads, 1) k_mlp_epoch(const __grid_con
         float g[4] = {0.0f, 0.0f, 0.0f, 0.0f};
         for (int g0 = 0; g0 < cnt; g0 += kGroupRows) {
             if (g0 > 0) cluster_sync();                        // every CTA's sums over the previous rows are done
+            if (S.failed) continue;                            // uniform: a barrier since the last wait
             // ---- phase F: rows row0 .. row0 + 15 of this minibatch
             const int row0 = g0 + kCtaRows * rank;
             if (t == 0) expect_bytes(&S.bar[0], kCluster * kRowBytes);
@@ -692,7 +693,7 @@ __global__ void __launch_bounds__(kEpochThreads, 1) k_mlp_epoch(const __grid_con
 
             // ---- phase G over these rows
             const int rows = min(kGroupRows, cnt - g0);
-            if (!S.failed && !wait_bar(&S.bar[0], row_phase & 1)) S.failed = 1;
+            if (!wait_bar(&S.bar[0], row_phase & 1)) S.failed = 1;
             ++row_phase;
             if (t < kIn) {
                 grad4<kIn>(g, &S.gx[0][t], rows, [&](int r) { return &S.gd[r >> 4].d1[r & 15][0]; });
@@ -719,7 +720,7 @@ __global__ void __launch_bounds__(kEpochThreads, 1) k_mlp_epoch(const __grid_con
             }
         }
         if (sums_loss && rank == 0) a.loss[step] = S.failed ? __int_as_float(0x7fc00000) : g[0] / (float)cnt;
-        if (t == 0) expect_bytes(&S.bar[1], kCluster * kRecord * 4);
+        if (t == 0 && !S.failed) expect_bytes(&S.bar[1], kCluster * kRecord * 4);
         const AdamArgs ad{nullptr, nullptr, nullptr, a.lr, a.b1, a.b2, a.eps, a.c1[step], a.c2[step]};
 #pragma unroll
         for (int u = 0; u < 4; ++u)
@@ -729,9 +730,17 @@ __global__ void __launch_bounds__(kEpochThreads, 1) k_mlp_epoch(const __grid_con
             }
         fence_async();
         __syncthreads();
-        if (t == 0) multicast(S.w + kRecord * rank, exch + xRec, kRecord * 4, &S.bar[1]);
-        if (!S.failed && !wait_bar(&S.bar[1], step & 1)) S.failed = 1;
+        // a CTA whose wait ran out sends nothing more, so the others' waits run
+        // out too; all still meet at every cluster barrier
+        if (!S.failed) {
+            if (t == 0) multicast(S.w + kRecord * rank, exch + xRec, kRecord * 4, &S.bar[1]);
+            if (!wait_bar(&S.bar[1], step & 1)) S.failed = 1;
+        }
         __syncthreads();
+    }
+    if (S.failed) {                                            // copies still on their way, again with a limit
+        wait_bar(&S.bar[0], (row_phase - 1) & 1);
+        wait_bar(&S.bar[1], (a.nsteps - 1) & 1);
     }
     cluster_sync();                                            // no CTA leaves while another still sends to it
 #pragma unroll
