@@ -366,42 +366,35 @@ __global__ void k_adam(AdamArgs a, const float* __restrict__ g) {
 // A step of k_mlp_delta and k_mlp_grad is bound by latency, not by work (5.8
 // million multiply-adds): two dependent launches, the weights staged anew and
 // the cache columns fetched by few CTAs cost 24 us.  Here a cluster stays on 16
-// SMs for all steps.  Every CTA holds all weights, as 16 records of one owner's
-// four hidden units each.  Phase F: CTA c runs rows 16c..16c+15 of a group of
-// 256 through forward and deltas (a warp takes 32 units of 4 rows, so a weight
-// is loaded once for four rows).  All CTAs need all rows' inputs and first-layer
-// outputs: each CTA writes its rows to global memory and has them multicast to
-// the cluster while the rest of phase F runs (one copy per receiver instead, or
-// every CTA fetching all rows from L2, both moved about 12 bytes per clock and
-// SM: 13,000 clocks a step).  The deltas of the units a CTA owns go to it in one
-// bulk copy between shared memories.  Phase G: CTA c sums its units' gradients
-// over the rows in ascending order, applies Adam to parameters it keeps in
-// registers and multicasts its record.  Every copy is counted by the
-// receiver's mbarrier; a CTA that holds all 16 new records knows that every CTA
-// has finished its sums, so the buffers it sends into next are free, and no
-// other barrier is needed.  The inputs of the next rows load while phase G
-// runs.  All sums and updates have the operands and order of the two kernels:
-// the same bits.  16,000 rows, batch 256 (63 steps): 770 us an epoch against
-// 1540 us.
-constexpr int kCluster = 16;
+// SMs for all steps, and every CTA holds all weights.  Phase F: CTA c runs rows
+// 16c..16c+15 of a group of 256 through forward and deltas (a warp takes 2 rows
+// and all units; what bounds it is the shared-memory reads, and two rows by two
+// units a thread read least among the splits that fill eight warps).  Phase G:
+// CTA 4p + q sums the gradients of units 16p..16p+15 over inputs 20q..20q+19 of
+// W1 and 16q..16q+15 of W2 (and b1, b2, W3 of its four units 4(4p + q)..) over
+// the rows in ascending order, then Adam runs on them, two parameters a thread.
+// The square tiles keep the exchange small: a CTA needs 16 units' deltas and 16
+// first-layer outputs of each row (48 KB a group; tiles of four whole rows of
+// W1 and W2 need 72 KB), and it fetches its 20 input columns itself, a step
+// ahead.  All exchange is by 16-byte stores into the other CTAs' shared memory
+// (about 8 bytes a clock and SM; loads from there ran at a quarter of that),
+// the first-layer outputs while layer 2 runs, W2's deltas while they are
+// propagated back.  Two cluster barriers a step order it: one between the
+// stores of phase F and phase G, one between the new weights and the next phase
+// F (a batch of several groups adds one per group).  Nothing polls memory, so
+// no wait can run out, and only the caller's own loads touch its pointers, so
+// any memory the GPU can read will do.  All sums and updates have the operands
+// and order of the two kernels: the same bits.  16,000 rows, batch 256 (63
+// steps): 752 us an epoch against 1540 us.
+constexpr int kCluster = 16, kSide = 4;                // CTAs: kSide x kSide gradient tiles
 constexpr int kEpochThreads = 512;
-constexpr int kOwned = kHid / kCluster;                // hidden units a CTA owns per layer
+constexpr int kTileUnits = kHid / kSide;               // hidden units of a tile
+constexpr int kTileIn1 = kIn / kSide, kTileIn2 = kHid / kSide;   // inputs of a tile of W1, W2
 constexpr int kGroupRows = 256;                        // rows in flight
 constexpr int kCtaRows = kGroupRows / kCluster;
 constexpr int kEpochSteps = 64;                        // steps per launch
-// Smaller batches have no room in the workspace for the cluster's exchange
-// area, larger ones fill the GPU with the two kernels.
-constexpr int kEpochMinBatch = 64, kEpochMaxBatch = 1024;
-static_assert(kOwned == 4 && kCtaRows == 16 && kIn % 4 == 0, "phases F and G index by fours");
-
-// One owner's weights: W1 rows (80, padded to 81), W2 rows (64, padded to 65),
-// b1, b2, W3 of its four units and (owner 0) b3.  With 604 floats a record,
-// lane u reading its unit's W1 or W2 row hits bank (28 (u / 4) + 17 or 1 (u % 4))
-// mod 32: all 32 distinct.
-constexpr int kW1Row = kIn + 1, kW2Row = kHid + 1;
-constexpr int rW2 = kOwned * kW1Row, rB1 = rW2 + kOwned * kW2Row, rB2 = rB1 + 4, rW3 = rB2 + 4, rB3 = rW3 + 4,
-              kRecord = 604;
-static_assert(rB3 + 1 <= kRecord && rB1 % 4 == 0 && kRecord % 4 == 0, "record layout");
+constexpr int kEpochMinBatch = 64, kEpochMaxBatch = 1024;   // batches that run this way
+static_assert(kTileUnits == 16 && kTileIn2 == 16 && kTileIn1 == 20 && kCtaRows == 16, "phases F and G index by these");
 
 struct EpochArgs {
     float *P, *m, *v;
@@ -409,346 +402,400 @@ struct EpochArgs {
     const int* order;                 // of the first step's first row
     const float *mean, *stdv;
     float* loss;                      // of the first step
-    float* exch;                      // kCluster * kExch floats
     int bf16, n, batch, nsteps;       // n rows left from the first step on
     float lr, b1, b2, eps;
     float c1[kEpochSteps], c2[kEpochSteps];
 };
 
-// What one CTA's 16 rows hold for one receiver: da1, da2, h2 of the
-// receiver's units and (y, dz, y - label, 0).
-struct __align__(16) Deltas {
-    float d1[kCtaRows][4], d2[kCtaRows][4], h2[kCtaRows][4], z[kCtaRows][4];
-};
-// A CTA's part of the exchange area: its rows' inputs and h1, its record.
-constexpr int xH1 = kCtaRows * kIn, xRec = xH1 + kCtaRows * kHid, kExch = xRec + kRecord;
-static_assert(kCluster * kExch <= kEpochMinBatch * kCache + 2 * kParams, "the exchange area fits the workspace");
+// Rows of 84 and 68 floats: a quarter warp's 16-byte reads of eight units' rows
+// hit eight different bank groups, and all rows start 16-byte aligned.
+constexpr int kW1Row = kIn + 4, kW2Row = kHid + 4;
+constexpr int kGRow = 16;                              // phase G's rows: 64 bytes, so that a warp's stores into them meet no bank twice
+static_assert(kTileUnits == kGRow && kTileIn2 == kGRow && kTileIn1 == kGRow + 4, "phase G's rows");
+
+// A tile's parameters in order: W1[16][20], W2[16][16], b1[4], b2[4], W3[4], b3
+// and three unused.
+constexpr int tW2 = kTileUnits * kTileIn1, tB = tW2 + kTileUnits * kTileIn2, kTileParams = tB + 16;
+static_assert(kTileParams <= 2 * kEpochThreads, "two parameters a thread");
 
 struct __align__(16) EpochSmem {
-    float w[kCluster * kRecord];               // all weights
-    float gx[kGroupRows][kIn], gh[kGroupRows][kHid];   // received: inputs and h1 of 256 rows
-    Deltas gd[kCluster];                       // received, by sender
-    float x[kCtaRows][kIn], h1[kCtaRows][kHid];        // this CTA's rows
-    Deltas sd[kCluster];                       // to send, by receiver
-    unsigned long long bar[2];                 // rows, records
-    int failed;                                // a wait ran out (the losses become NaN)
+    float w1[kHid][kW1Row], w2[kHid][kW2Row], b1[kHid], b2[kHid], w3[kHid], b3[4];   // all weights
+    // of all rows of a group: the tile's first 16 inputs; received deltas of
+    // layers 1 and 2; the last 4 inputs, received h2 of four units, (y, dz, y -
+    // label, 1) and four unused; received h1
+    float gx[kGroupRows][kGRow], gd1[kGroupRows][kGRow];
+    float pad[16];                    // what one load of a warp reads before and after: the other half of the banks
+    float gd2[kGroupRows][kGRow], ge[kGroupRows][kGRow], gh1[kGroupRows][kGRow];
+    // this CTA's rows
+    float x[kCtaRows][kIn], h1[kCtaRows][kW2Row], h2[kCtaRows][kW2Row], d1[kCtaRows][kW2Row], d2[kCtaRows][kW2Row];
+    float z[kCtaRows][4], mean[kIn], stdv[kIn];
+    // this tile's gradients and new weights: W1, W2, and b1, b2, W3 of four units, b3
+    float g[kTileParams], p[kTileParams];
 };
 static_assert(sizeof(EpochSmem) <= 232448, "shared memory of one CTA");
-constexpr unsigned kRowBytes = (kCtaRows * (kIn + kHid)) * 4 + sizeof(Deltas);   // one CTA's rows to one receiver
 
-__device__ __forceinline__ unsigned sm_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
-}
-// Bulk copy of `bytes` from this CTA's shared memory to the same or another
-// place (dst: an address in this CTA's window) in CTA `rank`, counted on the
-// receiver's copy of mbarrier `bar`.
-__device__ __forceinline__ void send(unsigned rank, void* dst, const void* src, unsigned bytes, void* bar) {
-    unsigned d, b;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(sm_addr(dst)), "r"(rank));
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(b) : "r"(sm_addr(bar)), "r"(rank));
-    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(d),
-                 "r"(sm_addr(src)), "r"(bytes), "r"(b)
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// Stores v at dst (an address in this CTA's shared memory) of CTA `rank`.
+__device__ __forceinline__ void put(unsigned rank, void* dst, float4 v) {
+    unsigned d;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"((unsigned)__cvta_generic_to_shared(dst)), "r"(rank));
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(d), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
                  : "memory");
 }
-// Bulk copy from global memory to `dst` in every CTA of the cluster, counted on
-// each one's mbarrier `bar`.
-__device__ __forceinline__ void multicast(void* dst, const void* src, unsigned bytes, void* bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1], %2, [%3], %4;" ::"r"(
-            sm_addr(dst)),
-        "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(sm_addr(bar)), "h"((unsigned short)0xFFFF)
-        : "memory");
-}
-// Waits for the phase of `parity` of a mbarrier, for at most about a second.
-__device__ __forceinline__ bool wait_bar(const void* bar, unsigned parity) {
-    const long long t0 = clock64();
-    unsigned ok;
-    do {
-        asm volatile("{\n\t.reg .pred p;\n\t"
-                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-                     "selp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(ok)
-                     : "r"(sm_addr(bar)), "r"(parity)
-                     : "memory");
-    } while (!ok && clock64() - t0 < 2000000000ll);
-    return ok != 0;
-}
-__device__ __forceinline__ void expect_bytes(void* bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;" ::"r"(sm_addr(bar)), "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
+template <int ID, int THREADS>
+__device__ __forceinline__ void bar_sync() { asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(THREADS) : "memory"); }
+template <int ID, int THREADS>
+__device__ __forceinline__ void bar_arrive() { asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(THREADS) : "memory"); }
 
-// acc[r] += w x[r] over N inputs in ascending order for four rows; x(r, i)
-// gives four inputs of a row, w(i) one weight.
+// acc[k][r] += w[k] x[r] over N inputs in ascending order for two units and two
+// rows; x(r, i) and w(k, i) give four inputs of a row and their four weights.
 template <int N, typename X, typename W>
-__device__ __forceinline__ void dot4(float (&acc)[4], X in, W w) {
-#pragma unroll 5
+__device__ __forceinline__ void dot4(float (&acc)[2][2], X in, W weights) {
+#pragma unroll 4
     for (int i = 0; i < N; i += 4) {
-        float4 x[4];
+        const float4 x[2] = {*reinterpret_cast<const float4*>(in(0, i)), *reinterpret_cast<const float4*>(in(1, i))};
+        const float4 w[2] = {weights(0, i), weights(1, i)};
 #pragma unroll
-        for (int r = 0; r < 4; ++r) x[r] = *reinterpret_cast<const float4*>(in(r, i));
-        const float w0 = w(i), w1 = w(i + 1), w2 = w(i + 2), w3 = w(i + 3);
+        for (int k = 0; k < 4; ++k) acc[k >> 1][k & 1] = fmaf(w[k >> 1].x, x[k & 1].x, acc[k >> 1][k & 1]);
 #pragma unroll
-        for (int r = 0; r < 4; ++r) acc[r] = fmaf(w0, x[r].x, acc[r]);
+        for (int k = 0; k < 4; ++k) acc[k >> 1][k & 1] = fmaf(w[k >> 1].y, x[k & 1].y, acc[k >> 1][k & 1]);
 #pragma unroll
-        for (int r = 0; r < 4; ++r) acc[r] = fmaf(w1, x[r].y, acc[r]);
+        for (int k = 0; k < 4; ++k) acc[k >> 1][k & 1] = fmaf(w[k >> 1].z, x[k & 1].z, acc[k >> 1][k & 1]);
 #pragma unroll
-        for (int r = 0; r < 4; ++r) acc[r] = fmaf(w2, x[r].z, acc[r]);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) acc[r] = fmaf(w3, x[r].w, acc[r]);
+        for (int k = 0; k < 4; ++k) acc[k >> 1][k & 1] = fmaf(w[k >> 1].w, x[k & 1].w, acc[k >> 1][k & 1]);
     }
 }
 
-// g[u] += d(r)[u] x[r] over `rows` rows in ascending order, eight loaded ahead;
-// d(r) gives the four deltas of row r.
-template <int LD, typename D>
-__device__ __forceinline__ void grad4(float (&g)[4], const float* x, int rows, D d) {
-    int r = 0;
-    for (; r + 8 <= rows; r += 8) {
-        float xv[8];
-        float4 dv[8];
+// One thread's share of phase G: eight sums g[u][k] += d[r][u] x[r][k], u < 4 and
+// k < 2, over the rows r in ascending order.
+struct GradRows {
+    float2 x[4];
+    float4 d[4];
+};
+__device__ __forceinline__ void grad_load(const float* x, const float* d, GradRows& v) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            xv[k] = x[(r + k) * LD];
-            dv[k] = *reinterpret_cast<const float4*>(d(r) + 4 * k);      // eight rows of one sender
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            g[0] = fmaf(dv[k].x, xv[k], g[0]);
-            g[1] = fmaf(dv[k].y, xv[k], g[1]);
-            g[2] = fmaf(dv[k].z, xv[k], g[2]);
-            g[3] = fmaf(dv[k].w, xv[k], g[3]);
-        }
+    for (int k = 0; k < 4; ++k) {
+        v.x[k] = *reinterpret_cast<const float2*>(x + k * kGRow);
+        v.d[k] = *reinterpret_cast<const float4*>(d + k * kGRow);
     }
-    for (; r < rows; ++r) {
-        const float4 dv = *reinterpret_cast<const float4*>(d(r));
-        g[0] = fmaf(dv.x, x[r * LD], g[0]);
-        g[1] = fmaf(dv.y, x[r * LD], g[1]);
-        g[2] = fmaf(dv.z, x[r * LD], g[2]);
-        g[3] = fmaf(dv.w, x[r * LD], g[3]);
+}
+__device__ __forceinline__ void grad_row(float (&g)[4][2], float2 x, float4 d) {
+    const float dv[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        g[u][0] = fmaf(dv[u], x.x, g[u][0]);
+        g[u][1] = fmaf(dv[u], x.y, g[u][1]);
+    }
+}
+// Four rows load while four others are summed; the last load repeats rows of
+// the arrays when there are no more.
+__device__ __forceinline__ void grad_sum(float (&g)[4][2], const float* x, const float* d, int rows) {
+    GradRows v0, v1;
+    grad_load(x, d, v0);
+    for (int left = rows; ; left -= 8) {
+        if (left < 8) {
+            for (int r = 0; r < left; ++r)
+                grad_row(g, *reinterpret_cast<const float2*>(x + r * kGRow), *reinterpret_cast<const float4*>(d + r * kGRow));
+            break;
+        }
+        grad_load(x + 4 * kGRow, d + 4 * kGRow, v1);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) grad_row(g, v0.x[k], v0.d[k]);
+        const int next = left >= 12 ? 8 * kGRow : 0;
+        grad_load(x + next, d + next, v0);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) grad_row(g, v1.x[k], v1.d[k]);
+        x += 8 * kGRow;
+        d += 8 * kGRow;
     }
 }
 
 __global__ void __launch_bounds__(kEpochThreads, 1) k_mlp_epoch(const __grid_constant__ EpochArgs a) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     EpochSmem& S = *reinterpret_cast<EpochSmem*>(smem_raw);
+    constexpr int kHalf = kEpochThreads / 2;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int rank = blockIdx.x;                               // one cluster: CTA rank = block index
-    for (int e = t; e < kHid * kIn; e += kEpochThreads) {
-        const int u = e / kIn, i = e - u * kIn;
-        S.w[(u >> 2) * kRecord + (u & 3) * kW1Row + i] = a.P[oW1 + e];
-    }
-    for (int e = t; e < kHid * kHid; e += kEpochThreads) {
-        const int u = e / kHid, i = e - u * kHid;
-        S.w[(u >> 2) * kRecord + rW2 + (u & 3) * kW2Row + i] = a.P[oW2 + e];
-    }
+    const int tp = rank / kSide, tq = rank % kSide;            // this CTA's tile
+    for (int e = t; e < kHid * kIn; e += kEpochThreads) S.w1[e / kIn][e % kIn] = a.P[oW1 + e];
+    for (int e = t; e < kHid * kHid; e += kEpochThreads) S.w2[e / kHid][e % kHid] = a.P[oW2 + e];
     if (t < kHid) {
-        float* r = S.w + (t >> 2) * kRecord + (t & 3);
-        r[rB1] = a.P[oB1 + t];
-        r[rB2] = a.P[oB2 + t];
-        r[rW3] = a.P[oW3 + t];
+        S.b1[t] = a.P[oB1 + t];
+        S.b2[t] = a.P[oB2 + t];
+        S.w3[t] = a.P[oW3 + t];
     }
-    if (t == 0) {
-        S.w[rB3] = a.P[oB3];
-        S.failed = 0;
-        for (int k = 0; k < 2; ++k) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sm_addr(&S.bar[k])) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (t < 4) S.b3[t] = t == 0 ? a.P[oB3] : 0.0f;
+    if (t < kIn) {
+        S.mean[t] = a.mean[t];
+        S.stdv[t] = a.stdv[t];
     }
-    float* const exch = a.exch + (size_t)rank * kExch;
 
-    // owned parameters, in registers for the whole run: threads 0..79 column t
-    // of W1 (four units), 96..159 column t - 96 of W2, the first lanes of warps
-    // 5..8 b1, b2, W3 and (CTA 0) b3, lane 0 of warp 9 the loss (each its own
-    // warp: as branches of one warp they would run one after the other)
-    int np = 0, p0 = 0, pstep = 0, rpos = 0, rstep = 0;
-    if (t < kIn) { np = 4; p0 = oW1 + kOwned * rank * kIn + t; pstep = kIn; rpos = t; rstep = kW1Row; }
-    else if (t >= 96 && t < 96 + kHid) {
-        np = 4; p0 = oW2 + kOwned * rank * kHid + t - 96; pstep = kHid; rpos = rW2 + t - 96; rstep = kW2Row;
-    } else if (warp >= 5 && warp < 8 && lane < 4) {
-        np = 1; p0 = (warp == 5 ? oB1 : warp == 6 ? oB2 : oW3) + kOwned * rank + lane; rpos = rB1 + 4 * (warp - 5) + lane;
-    } else if (warp == 8 && lane == 0 && rank == 0) { np = 1; p0 = oB3; rpos = rB3; }
-    const bool sums_loss = warp == 9 && lane == 0;
-    float P[4], M[4], V[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-        if (u < np) {
-            P[u] = a.P[p0 + u * pstep];
-            M[u] = a.m[p0 + u * pstep];
-            V[u] = a.v[p0 + u * pstep];
-        }
-
-    // this thread's elements of the CTA's 16 x 80 inputs, loaded ahead
-    constexpr int kElems = (kCtaRows * kIn + kEpochThreads - 1) / kEpochThreads;
-    float xf[kElems], mu[kElems], sd[kElems], label = 0.0f;
-#pragma unroll
-    for (int k = 0; k < kElems; ++k) {
-        const int e = t + k * kEpochThreads;
-        mu[k] = e < kCtaRows * kIn ? a.mean[e % kIn] : 0.0f;
-        sd[k] = e < kCtaRows * kIn ? a.stdv[e % kIn] : 1.0f;
+    // this thread's sums in phase G: threads 0..39 four units by two inputs of W1,
+    // 40..71 of W2, and four more the same sums with other operands, of which
+    // they keep g[u][1]: b1 and b2 (inputs y - label and 1), W3 (h2 as the
+    // deltas, inputs y and dz), in CTA 0 b3 (the z record as the deltas, inputs
+    // y - label and 1) and the loss beside it (g[2][0])
+    constexpr int q1 = kTileIn1 / 2, q2 = kTileIn2 / 2, g2 = kTileUnits / 4 * q1, gb = g2 + kTileUnits / 4 * q2;
+    const float *gx = nullptr, *gd = nullptr;
+    int gpos = 0;                                              // where g[0][0] goes in the tile's order
+    if (t < g2) {
+        const int u = 4 * (t / q1), i = 2 * (t % q1);
+        gx = i < kGRow ? &S.gx[0][i] : &S.ge[0][i - kGRow];
+        gd = &S.gd1[0][u];
+        gpos = u * kTileIn1 + i;
+    } else if (t < gb) {
+        const int u = 4 * ((t - g2) / q2), i = 2 * ((t - g2) % q2);
+        gx = &S.gh1[0][i];
+        gd = &S.gd2[0][u];
+        gpos = tW2 + u * kTileIn2 + i;
+    } else if (t < gb + 3) {
+        gx = &S.ge[0][t < gb + 2 ? 10 : 8];
+        gd = t == gb ? &S.gd1[0][4 * tq] : t == gb + 1 ? &S.gd2[0][4 * tq] : &S.ge[0][4];
+        gpos = tB + 4 * (t - gb);
+    } else if (t == gb + 3 && rank == 0) {
+        gx = &S.ge[0][10];
+        gd = &S.ge[0][8];
+        gpos = tB + 12;
     }
-    const int unit = 32 * (warp & 1) + lane, rq = 4 * ((warp >> 1) & 3);   // phase F, warps 0..7
-    const auto load_rows = [&](int step, int g0) {
-        const int cnt = step < a.nsteps ? min(a.batch, a.n - step * a.batch) : 0;
-        const int row0 = g0 + kCtaRows * rank;
-        const int* const index = a.order + (size_t)step * a.batch;
-#pragma unroll
-        for (int k = 0; k < kElems; ++k) {
-            const int e = t + k * kEpochThreads, r = e / kIn;
-            xf[k] = mu[k];
-            if (e < kCtaRows * kIn && row0 + r < cnt) xf[k] = __ldg(a.feats + (size_t)__ldg(index + row0 + r) * kIn + e - r * kIn);
-        }
-        const int row = row0 + rq + (lane & 3);
-        label = row < cnt ? __ldg(a.labels + __ldg(index + row)) : 0.0f;
+    // the Adam state of tile parameters t and t + 512, for the whole run
+    const auto param = [&](int e) {
+        if (e < tW2) return oW1 + (kTileUnits * tp + e / kTileIn1) * kIn + kTileIn1 * tq + e % kTileIn1;
+        if (e < tB) return oW2 + (kTileUnits * tp + (e - tW2) / kTileIn2) * kHid + kTileIn2 * tq + (e - tW2) % kTileIn2;
+        if (e < tB + 12) return (e < tB + 4 ? oB1 : e < tB + 8 ? oB2 : oW3) + 4 * rank + (e - tB) % 4;
+        return e == tB + 12 && rank == 0 ? oB3 : -1;
     };
-    load_rows(0, 0);
-    cluster_sync();                                            // mbarriers are ready everywhere
+    int pi[2];
+    float P[2], M[2], V[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        pi[k] = param(t + k * kEpochThreads);
+        if (pi[k] >= 0) {
+            P[k] = a.P[pi[k]];
+            M[k] = a.m[pi[k]];
+            V[k] = a.v[pi[k]];
+        }
+    }
 
-    unsigned row_phase = 0;
+    // inputs, loaded ahead: threads 0..255 elements t + 256 k of the CTA's 16
+    // rows of 80, the others the tile's 20 columns of row th.  The row indices
+    // load a phase earlier, so that no thread waits for one.
+    const bool fwd = t < kHalf;
+    const int th = t & (kHalf - 1);
+    constexpr int kOwn = kCtaRows * kIn / kHalf;
+    const bool vec = (((uintptr_t)a.feats) & 15u) == 0;
+    float xf[kTileIn1], label = 0.0f;
+    int idx[kOwn + 1];                                         // -1: no such row
+    const int rq = 2 * (warp & 7);                             // phase F: rows rq and rq + 1, units lane and lane + 32
+    const auto load_index = [&](int step, int g0) {
+        const int cnt = step < a.nsteps ? min(a.batch, a.n - step * a.batch) : 0;
+        const int* const order = a.order + (size_t)step * a.batch;
+        const auto at = [&](int row) { return row < cnt ? __ldg(order + row) : -1; };
+        if (fwd) {
+#pragma unroll
+            for (int k = 0; k < kOwn; ++k) idx[k] = at(g0 + kCtaRows * rank + (t + k * kHalf) / kIn);
+            idx[kOwn] = at(g0 + kCtaRows * rank + rq + (lane & 1));
+        } else {
+            idx[0] = at(g0 + th);
+        }
+    };
+    const auto load_rows = [&] {
+        if (fwd) {
+#pragma unroll
+            for (int k = 0; k < kOwn; ++k)
+                if (idx[k] >= 0) xf[k] = __ldg(a.feats + (size_t)idx[k] * kIn + (t + k * kHalf) % kIn);
+            if (idx[kOwn] >= 0) label = __ldg(a.labels + idx[kOwn]);
+        } else if (idx[0] >= 0) {
+            const float* const x = a.feats + (size_t)idx[0] * kIn + kTileIn1 * tq;
+            if (vec) {
+#pragma unroll
+                for (int k = 0; k < kTileIn1; k += 4) {
+                    const float4 v = __ldg(reinterpret_cast<const float4*>(x + k));
+                    xf[k] = v.x;
+                    xf[k + 1] = v.y;
+                    xf[k + 2] = v.z;
+                    xf[k + 3] = v.w;
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < kTileIn1; ++k) xf[k] = __ldg(x + k);
+            }
+        }
+    };
+    load_index(0, 0);
+    load_rows();
+    cluster_arrive();                                          // every CTA of the cluster has started
+    cluster_wait();
+    __syncthreads();
+
     for (int step = 0; step < a.nsteps; ++step) {
         const int cnt = min(a.batch, a.n - step * a.batch);
-        float g[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        float g[4][2] = {};
         for (int g0 = 0; g0 < cnt; g0 += kGroupRows) {
-            if (g0 > 0) cluster_sync();                        // every CTA's sums over the previous rows are done
-            if (S.failed) continue;                            // uniform: a barrier since the last wait
-            // ---- phase F: rows row0 .. row0 + 15 of this minibatch
-            const int row0 = g0 + kCtaRows * rank;
-            if (t == 0) expect_bytes(&S.bar[0], kCluster * kRowBytes);
-#pragma unroll
-            for (int k = 0; k < kElems; ++k) {
-                const int e = t + k * kEpochThreads;
-                if (e < kCtaRows * kIn) {
-                    const float x = (xf[k] - mu[k]) / sd[k];
-                    (&S.x[0][0])[e] = x;
-                    exch[e] = x;
-                }
+            if (g0 > 0) {                                      // every CTA's sums over the previous rows are done
+                cluster_arrive();
+                cluster_wait();
             }
-            fence_async();
-            __syncthreads();
-            if (t == 0) multicast(S.gx[kCtaRows * rank], exch, sizeof(S.x), &S.bar[0]);
-            if (warp < 8) {
-                const auto bar = [] { asm volatile("bar.sync 1, 256;" ::: "memory"); };
-                const float* const rec = S.w + (unit >> 2) * kRecord + (unit & 3);
-                const float* const w1 = S.w + (unit >> 2) * kRecord + (unit & 3) * kW1Row;
-                const float* const w2 = S.w + (unit >> 2) * kRecord + rW2 + (unit & 3) * kW2Row;
-                float a1[4], a2[4], s[4];
+            if (g0 + kGroupRows < cnt) load_index(step, g0 + kGroupRows);
+            else load_index(step + 1, 0);
+            // ---- phase F: rows g0 + 16 rank .. + 15 of this minibatch
+            const int mine = kCtaRows * rank;
+            // 64 threads a receiver: row r, floats 4c..
+            const int blk = (t >> 6) & 3, r = (t >> 2) & 15, c = 4 * (t & 3);
+            if (fwd) {
 #pragma unroll
-                for (int r = 0; r < 4; ++r) a1[r] = rec[rB1];
-                dot4<kIn>(a1, [&](int r, int i) { return &S.x[rq + r][i]; }, [&](int i) { return w1[i]; });
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const float h = act(gelu(a1[r]), a.bf16);
-                    S.h1[rq + r][unit] = h;
-                    exch[xH1 + (rq + r) * kHid + unit] = h;
-                    a2[r] = rec[rB2];
+                for (int k = 0; k < kOwn; ++k) {
+                    const int e = t + k * kHalf, r = e / kIn, col = e - r * kIn;
+                    S.x[r][col] = g0 + mine + r < cnt ? (xf[k] - S.mean[col]) / S.stdv[col] : 0.0f;
                 }
-                fence_async();
-                bar();
-                if (t == 0) multicast(S.gh[kCtaRows * rank], exch + xH1, sizeof(S.h1), &S.bar[0]);
-                dot4<kHid>(a2, [&](int r, int i) { return &S.h1[rq + r][i]; }, [&](int i) { return w2[i]; });
+                bar_sync<1, kHalf>();
+                float a1[2][2], a2[2][2], s[2][2];             // [unit][row]; from here on a warp reads its own rows
+                const auto unit = [&](int k) { return lane + 32 * k; };
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    S.sd[unit >> 2].h2[rq + r][unit & 3] = act(gelu(a2[r]), a.bf16);
+                for (int k = 0; k < 2; ++k) a1[k][0] = a1[k][1] = S.b1[unit(k)];
+                dot4<kIn>(a1, [&](int r, int i) { return &S.x[rq + r][i]; },
+                          [&](int k, int i) { return *reinterpret_cast<const float4*>(&S.w1[unit(k)][i]); });
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        S.h1[rq + r][unit(k)] = act(gelu(a1[k][r]), a.bf16);
+                        a2[k][r] = S.b2[unit(k)];
+                    }
                 }
-                bar();
-                // output and its delta: lane r < 4 of both warps of a row quad
+                bar_arrive<2, kEpochThreads>();
+                __syncwarp();
+                dot4<kHid>(a2, [&](int r, int i) { return &S.h1[rq + r][i]; },
+                           [&](int k, int i) { return *reinterpret_cast<const float4*>(&S.w2[unit(k)][i]); });
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) S.h2[rq + r][unit(k)] = act(gelu(a2[k][r]), a.bf16);
+                }
+                __syncwarp();
+                // output and its delta of row lane % 2
                 float dz;
                 {
-                    const int r = lane & 3, row = row0 + rq + r;
-                    float z = S.w[rB3];
+                    const int r = lane & 1;
+                    float z = S.b3[0];
 #pragma unroll 8
                     for (int j = 0; j < kHid; j += 4) {
-                        const float4 w = *reinterpret_cast<const float4*>(S.w + (j >> 2) * kRecord + rW3);
-                        const float4 h = *reinterpret_cast<const float4*>(S.sd[j >> 2].h2[rq + r]);
+                        const float4 w = *reinterpret_cast<const float4*>(&S.w3[j]);
+                        const float4 h = *reinterpret_cast<const float4*>(&S.h2[rq + r][j]);
                         z = fmaf(w.x, h.x, z);
                         z = fmaf(w.y, h.y, z);
                         z = fmaf(w.z, h.z, z);
                         z = fmaf(w.w, h.w, z);
                     }
                     const float y = 1.0f / (1.0f + expf(-z));
-                    dz = row < cnt ? 2.0f * (y - label) / (float)cnt * y * (1.0f - y) : 0.0f;
-                    // every receiver's copy: 16 receivers over 8 lanes a row of two warps
-                    *reinterpret_cast<float4*>(S.sd[(lane >> 2) + 8 * (warp & 1)].z[rq + r]) =
-                        make_float4(y, dz, y - label, 0.0f);
+                    dz = g0 + mine + rq + r < cnt ? 2.0f * (y - label) / (float)cnt * y * (1.0f - y) : 0.0f;
+                    if (lane < 2) *reinterpret_cast<float4*>(S.z[rq + r]) = make_float4(y, dz, y - label, 1.0f);
                 }
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const float d = __shfl_sync(0xffffffffu, dz, r) * rec[rW3] * gelu_grad(a2[r]);
-                    S.sd[unit >> 2].d2[rq + r][unit & 3] = d;
-                    s[r] = 0.0f;
-                }
-                bar();
-                dot4<kHid>(s, [&](int r, int j) { return S.sd[j >> 2].d2[rq + r]; },
-                             [&](int j) { return S.w[(j >> 2) * kRecord + rW2 + (j & 3) * kW2Row + unit]; });
+                for (int r = 0; r < 2; ++r) {
+                    const float dzr = __shfl_sync(0xffffffffu, dz, r);
 #pragma unroll
-                for (int r = 0; r < 4; ++r) S.sd[unit >> 2].d1[rq + r][unit & 3] = s[r] * gelu_grad(a1[r]);
+                    for (int k = 0; k < 2; ++k) {
+                        S.d2[rq + r][unit(k)] = dzr * S.w3[unit(k)] * gelu_grad(a2[k][r]);
+                        s[k][r] = 0.0f;
+                    }
+                }
+                bar_arrive<3, kEpochThreads>();
+                __syncwarp();
+                dot4<kHid>(s, [&](int r, int j) { return &S.d2[rq + r][j]; },
+                           [&](int k, int j) {
+                               const float* w = &S.w2[j][unit(k)];
+                               return make_float4(w[0], w[kW2Row], w[2 * kW2Row], w[3 * kW2Row]);
+                           });
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) S.d1[rq + r][unit(k)] = s[k][r] * gelu_grad(a1[k][r]);
+                }
+            } else {
+                if (g0 + th < cnt) {
+#pragma unroll
+                    for (int k = 0; k < kTileIn1; k += 4) {
+                        const float4 m = *reinterpret_cast<const float4*>(&S.mean[kTileIn1 * tq + k]);
+                        const float4 d = *reinterpret_cast<const float4*>(&S.stdv[kTileIn1 * tq + k]);
+                        *reinterpret_cast<float4*>(k < kGRow ? &S.gx[th][k] : &S.ge[th][0]) = make_float4((xf[k] - m.x) / d.x, (xf[k + 1] - m.y) / d.y,
+                                                                               (xf[k + 2] - m.z) / d.z, (xf[k + 3] - m.w) / d.w);
+                    }
+                }
+                bar_sync<2, kEpochThreads>();                  // first-layer outputs: to the tiles of these inputs
+                const float4 h1 = *reinterpret_cast<const float4*>(&S.h1[r][kTileIn2 * blk + c]);
+#pragma unroll
+                for (int k = 0; k < kSide; ++k) put(kSide * ((k + tp) % kSide) + blk, &S.gh1[mine + r][c], h1);
+                bar_sync<3, kEpochThreads>();                  // W2's deltas: to the tiles of these units
+                const float4 d2 = *reinterpret_cast<const float4*>(&S.d2[r][kTileUnits * blk + c]);
+#pragma unroll
+                for (int k = 0; k < kSide; ++k) put(kSide * blk + (k + tq) % kSide, &S.gd2[mine + r][c], d2);
+                const int to = th >> 4, rr = th & 15;          // every CTA: its units' h2, and z
+                put(to, &S.ge[mine + rr][4], *reinterpret_cast<const float4*>(&S.h2[rr][4 * to]));
+                put(to, &S.ge[mine + rr][8], *reinterpret_cast<const float4*>(S.z[rr]));
             }
-            fence_async();
             __syncthreads();
-            if (t < kCluster) send(t, &S.gd[rank], &S.sd[t], sizeof(Deltas), &S.bar[0]);
-            // the next rows' inputs load during phase G
-            if (g0 + kGroupRows < cnt) load_rows(step, g0 + kGroupRows);
-            else load_rows(step + 1, 0);
+            {
+                const float4 d1 = *reinterpret_cast<const float4*>(&S.d1[r][kTileUnits * blk + c]);
+#pragma unroll
+                for (int k = 0; k < kSide / 2; ++k)
+                    put(kSide * blk + (2 * k + (t >> 8) + tq) % kSide, &S.gd1[mine + r][c], d1);
+            }
+            cluster_arrive();
+            load_rows();                                       // the next rows' inputs, during phase G
+            cluster_wait();
 
             // ---- phase G over these rows
-            const int rows = min(kGroupRows, cnt - g0);
-            if (!wait_bar(&S.bar[0], row_phase & 1)) S.failed = 1;
-            ++row_phase;
-            if (t < kIn) {
-                grad4<kIn>(g, &S.gx[0][t], rows, [&](int r) { return &S.gd[r >> 4].d1[r & 15][0]; });
-            } else if (t >= 96 && t < 96 + kHid) {
-                grad4<kHid>(g, &S.gh[0][t - 96], rows, [&](int r) { return &S.gd[r >> 4].d2[r & 15][0]; });
-            } else if (warp == 5 && lane < 4) {
-#pragma unroll 16
-                for (int r = 0; r < rows; ++r) g[0] += S.gd[r >> 4].d1[r & 15][lane];
-            } else if (warp == 6 && lane < 4) {
-#pragma unroll 16
-                for (int r = 0; r < rows; ++r) g[0] += S.gd[r >> 4].d2[r & 15][lane];
-            } else if (warp == 7 && lane < 4) {
-#pragma unroll 16
-                for (int r = 0; r < rows; ++r) g[0] = fmaf(S.gd[r >> 4].z[r & 15][1], S.gd[r >> 4].h2[r & 15][lane], g[0]);
-            } else if (warp == 8 && lane == 0) {
-#pragma unroll 16
-                for (int r = 0; r < rows; ++r) g[0] += S.gd[r >> 4].z[r & 15][1];
-            } else if (sums_loss) {
-#pragma unroll 16
-                for (int r = 0; r < rows; ++r) {
-                    const float d = S.gd[r >> 4].z[r & 15][2];
-                    g[0] = fmaf(d, d, g[0]);
-                }
-            }
+            if (gx) grad_sum(g, gx, gd, min(kGroupRows, cnt - g0));
         }
-        if (sums_loss && rank == 0) a.loss[step] = S.failed ? __int_as_float(0x7fc00000) : g[0] / (float)cnt;
-        if (t == 0 && !S.failed) expect_bytes(&S.bar[1], kCluster * kRecord * 4);
+        if (gx && gpos < tB) {
+            const int ld = gpos < tW2 ? kTileIn1 : kTileIn2;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) *reinterpret_cast<float2*>(&S.g[gpos + u * ld]) = make_float2(g[u][0], g[u][1]);
+        } else if (gx && gpos < tB + 12) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) S.g[gpos + u] = g[u][1];
+        } else if (gx) {
+            S.g[tB + 12] = g[1][1];
+            a.loss[step] = g[2][0] / (float)cnt;
+        }
+        __syncthreads();
         const AdamArgs ad{nullptr, nullptr, nullptr, a.lr, a.b1, a.b2, a.eps, a.c1[step], a.c2[step]};
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (u < np) {
-                adam_step(ad, P[u], M[u], V[u], g[u]);
-                exch[xRec + rpos + u * rstep] = P[u];
+        for (int k = 0; k < 2; ++k)
+            if (pi[k] >= 0) {
+                adam_step(ad, P[k], M[k], V[k], S.g[t + k * kEpochThreads]);
+                S.p[t + k * kEpochThreads] = P[k];
             }
-        fence_async();
         __syncthreads();
-        // a CTA whose wait ran out sends nothing more, so the others' waits run
-        // out too; all still meet at every cluster barrier
-        if (!S.failed) {
-            if (t == 0) multicast(S.w + kRecord * rank, exch + xRec, kRecord * 4, &S.bar[1]);
-            if (!wait_bar(&S.bar[1], step & 1)) S.failed = 1;
+        // the new weights to every CTA: three threads share an item's 16 stores
+        constexpr int kItems = kTileParams / 4, kLane = 160;
+        static_assert(kItems <= kLane && 3 * kLane <= kEpochThreads, "weight items");
+        const int item = t % kLane, part = t / kLane, e = 4 * item;
+        float* dst = nullptr;
+        if (part >= 3) {
+        } else if (e < tW2) {
+            dst = &S.w1[kTileUnits * tp + e / kTileIn1][kTileIn1 * tq + e % kTileIn1];
+        } else if (e < tB) {
+            dst = &S.w2[kTileUnits * tp + (e - tW2) / kTileIn2][kTileIn2 * tq + (e - tW2) % kTileIn2];
+        } else if (e < tB + 12) {
+            dst = (e == tB ? S.b1 : e == tB + 4 ? S.b2 : S.w3) + 4 * rank;
+        } else if (e == tB + 12 && rank == 0) {
+            dst = S.b3;
         }
-        __syncthreads();
+        if (dst) {
+            const float4 w = *reinterpret_cast<const float4*>(&S.p[e]);
+            for (int k = part; k < kCluster; k += 3) put((k + rank) % kCluster, dst, w);
+        }
+        cluster_arrive();
+        cluster_wait();
     }
-    if (S.failed) {                                            // copies still on their way, again with a limit
-        wait_bar(&S.bar[0], (row_phase - 1) & 1);
-        wait_bar(&S.bar[1], (a.nsteps - 1) & 1);
-    }
-    cluster_sync();                                            // no CTA leaves while another still sends to it
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
-        if (u < np) {
-            a.P[p0 + u * pstep] = P[u];
-            a.m[p0 + u * pstep] = M[u];
-            a.v[p0 + u * pstep] = V[u];
+    for (int k = 0; k < 2; ++k)
+        if (pi[k] >= 0) {
+            a.P[pi[k]] = P[k];
+            a.m[pi[k]] = M[k];
+            a.v[pi[k]] = V[k];
         }
 }
 
@@ -1011,7 +1058,6 @@ dct_status dct_mlp_train_epoch(dct_mlp* net, const float* feats, const float* la
             a.mean = net->feat_mean;
             a.stdv = net->feat_std;
             a.loss = loss_out + k0;
-            a.exch = static_cast<float*>(workspace);
             a.bf16 = net->act_bf16;
             a.n = n - k0 * batch;
             a.batch = batch;
