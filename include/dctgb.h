@@ -387,8 +387,8 @@ dct_status dct_mlp_adam(dct_mlp* net, const float* grad, float lr, float beta1, 
 /* One epoch of minibatch training: for each consecutive `batch` rows of
  * order[0..n) (device int32, a permutation chosen by the caller) a
  * loss_grad + adam step (beta1 0.9, beta2 0.999, eps 1e-8) with the same
- * arithmetic (up to batch 1024 a run of steps in one launch, beyond that two
- * launches per minibatch).  batch in 1..2^20, lr > 0.  loss_out: device
+ * arithmetic (up to 64 steps in one launch; step by step on a device
+ * that cannot hold a cluster of 16 CTAs).  batch in 1..2^20, lr > 0.  loss_out: device
  * float[ceil(n / batch)].  workspace: dct_mlp_workspace_bytes(batch) +
  * DCT_MLP_PARAMS floats. */
 dct_status dct_mlp_train_epoch(dct_mlp* net, const float* feats, const float* labels, const int32_t* order, int n,

@@ -3,7 +3,7 @@
 // (fixed-order) minibatch sums, and Adam.  The network is tiny (9409
 // parameters), so it runs on plain FMA units: one warp per sample for
 // inference, one cluster of 16 CTAs for a run of training steps; single
-// gradients and the smallest and largest batches use one warp per minibatch
+// gradients (and epochs where no cluster of 16 fits) use one warp per minibatch
 // row for the forward and delta pass and one thread per parameter for the
 // gradient sums (in tiles that stage the minibatch in shared memory) and the
 // update.
@@ -232,7 +232,7 @@ constexpr int kGradCtas = kW1Tiles + kW2Tiles + 3;
 constexpr int kGradThreads = kGradUnits * kIn;               // the widest tile
 static_assert(kHid % kGradUnits == 0 && kGradThreads >= kHid + 2, "gradient tiling");
 
-// Adam step for one parameter (k_adam and the fused gradient kernel)
+// Adam step for one parameter (k_adam and the training cluster)
 struct AdamArgs {
     float* P;
     float* m;
@@ -247,17 +247,10 @@ __device__ __forceinline__ void adam_step(const AdamArgs& a, float& P, float& m,
     v = fmaf(__fmul_rn(1.0f - a.b2, gi), gi, __fmul_rn(a.b2, v));
     P = __fsub_rn(P, __fdiv_rn(__fmul_rn(a.lr, __fmul_rn(m, a.c1)), __fadd_rn(__fsqrt_rn(__fmul_rn(v, a.c2)), a.eps)));
 }
-__device__ __forceinline__ void adam_update(const AdamArgs& a, int p, float gi) {
-    adam_step(a, a.P[p], a.m[p], a.v[p], gi);
-}
 
-// ADAM: also apply the Adam step to each parameter as soon as its sum is
-// final (each parameter belongs to one thread; nothing in this kernel reads
-// the parameters), saving the separate update launch of a training step.
-template <bool ADAM>
 __global__ void __launch_bounds__(kGradThreads)
 k_mlp_grad(const float* __restrict__ cache, const float* __restrict__ labels, const int* __restrict__ index,
-           int batch, float* __restrict__ grad, float* __restrict__ loss, AdamArgs adam) {
+           int batch, float* __restrict__ grad, float* __restrict__ loss) {
     __shared__ __align__(16) float sm[kGradRows * (kGradUnits + kIn)];
     const int t = threadIdx.x;
     const int blk = blockIdx.x;
@@ -348,16 +341,13 @@ k_mlp_grad(const float* __restrict__ cache, const float* __restrict__ labels, co
     } else if (t == kHid + 1) {
         *loss = g / (float)batch;
     }
-    if (p >= 0) {
-        grad[p] = g;
-        if (ADAM) adam_update(adam, p, g);
-    }
+    if (p >= 0) grad[p] = g;
 }
 
 __global__ void k_adam(AdamArgs a, const float* __restrict__ g) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= kParams) return;
-    adam_update(a, p, g[p]);
+    adam_step(a, a.P[p], a.m[p], a.v[p], g[p]);
 }
 
 // ---------------------------------------------------------------------------
@@ -384,8 +374,10 @@ __global__ void k_adam(AdamArgs a, const float* __restrict__ g) {
 // F (a batch of several groups adds one per group).  Nothing polls memory, so
 // no wait can run out, and only the caller's own loads touch its pointers, so
 // any memory the GPU can read will do.  All sums and updates have the operands
-// and order of the two kernels: the same bits.  16,000 rows, batch 256 (63
-// steps): 752 us an epoch against 1540 us.
+// and order of k_mlp_delta, k_mlp_grad and k_adam: the same bits.  16,000 rows, batch 256 (63
+// steps): 752 us an epoch against 1540 us.  It runs every batch size: 24 steps,
+// us, this way against two launches a step: batch 1 227 / 315, 32 236 / 363, 64 246 /
+// 364, 512 531 / 835, 1024 977 / 1398, 4096 3652 / 4737, 65536 64056 / 101761.
 constexpr int kCluster = 16, kSide = 4;                // CTAs: kSide x kSide gradient tiles
 constexpr int kEpochThreads = 512;
 constexpr int kTileUnits = kHid / kSide;               // hidden units of a tile
@@ -393,7 +385,6 @@ constexpr int kTileIn1 = kIn / kSide, kTileIn2 = kHid / kSide;   // inputs of a 
 constexpr int kGroupRows = 256;                        // rows in flight
 constexpr int kCtaRows = kGroupRows / kCluster;
 constexpr int kEpochSteps = 64;                        // steps per launch
-constexpr int kEpochMinBatch = 64, kEpochMaxBatch = 1024;   // batches that run this way
 static_assert(kTileUnits == 16 && kTileIn2 == 16 && kTileIn1 == 20 && kCtaRows == 16, "phases F and G index by these");
 
 struct EpochArgs {
@@ -908,14 +899,12 @@ static AdamArgs next_adam_step(dct_mlp* net, float lr, float beta1, float beta2,
 
 // one minibatch: forward and deltas (one warp per row, 8 rows per CTA,
 // weights staged once per CTA), then one CTA per gradient tile
-template <bool ADAM>
-static cudaError_t launch_train_step(const dct_mlp* net, const float* feats, const float* labels, const int* index,
-                                     int batch, float* grad, float* loss, void* workspace, AdamArgs adam,
-                                     cudaStream_t s) {
+static cudaError_t launch_loss_grad(const dct_mlp* net, const float* feats, const float* labels, const int* index,
+                                    int batch, float* grad, float* loss, void* workspace, cudaStream_t s) {
     float* cache = static_cast<float*>(workspace);
     k_mlp_delta<<<(batch + kDeltaRows - 1) / kDeltaRows, kDeltaRows * 32, 0, s>>>(
         net->params, feats, labels, index, net->feat_mean, net->feat_std, net->act_bf16, batch, cache);
-    k_mlp_grad<ADAM><<<kGradCtas, kGradThreads, 0, s>>>(cache, labels, index, batch, grad, loss, adam);
+    k_mlp_grad<<<kGradCtas, kGradThreads, 0, s>>>(cache, labels, index, batch, grad, loss);
     return cudaGetLastError();
 }
 
@@ -1006,8 +995,8 @@ dct_status dct_mlp_loss_grad(const dct_mlp* net, const float* feats, const float
         return fail(DCT_ERR_INVALID_ARG, "null pointer");
     if (batch < 1 || batch > (1 << 20)) return fail(DCT_ERR_INVALID_ARG, "batch must be 1..2^20");
     if (((uintptr_t)workspace) & 15u) return fail(DCT_ERR_INVALID_ARG, "workspace must be 16-byte aligned");
-    cudaError_t e = launch_train_step<false>(net, feats, labels, index, batch, grad_out, loss_out, workspace,
-                                             AdamArgs{}, (cudaStream_t)stream);
+    cudaError_t e = launch_loss_grad(net, feats, labels, index, batch, grad_out, loss_out, workspace,
+                                     (cudaStream_t)stream);
     return e == cudaSuccess ? DCT_OK : cuda_fail(e, "gradient launch");
 }
 
@@ -1030,11 +1019,11 @@ dct_status dct_mlp_train_epoch(dct_mlp* net, const float* feats, const float* la
     if (n < 1 || batch < 1 || batch > (1 << 20)) return fail(DCT_ERR_INVALID_ARG, "n >= 1 and batch in 1..2^20");
     if (!adam_params_ok(lr, 0.9f, 0.999f, 1e-8f)) return fail(DCT_ERR_INVALID_ARG, "learning rate must be > 0");
     if (((uintptr_t)workspace) & 15u) return fail(DCT_ERR_INVALID_ARG, "workspace must be 16-byte aligned");
-    // batches that one cluster handles: runs of steps in one launch
+    // runs of steps in one launch, where the device can hold the cluster
     cudaStream_t st_ = (cudaStream_t)stream;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at;
-    if (batch >= kEpochMinBatch && batch <= kEpochMaxBatch && epoch_cluster_config(cfg, at, st_)) {
+    if (epoch_cluster_config(cfg, at, st_)) {
         const int steps = (n + batch - 1) / batch;
         for (int k0 = 0; k0 < steps; k0 += kEpochSteps) {
             EpochArgs a;
@@ -1066,14 +1055,13 @@ dct_status dct_mlp_train_epoch(dct_mlp* net, const float* feats, const float* la
         }
         return DCT_OK;
     }
-    // per minibatch: the delta kernel, then the gradient sums with the Adam
-    // step fused (same arithmetic as dct_mlp_loss_grad + dct_mlp_adam)
+    // elsewhere step by step, as dct_mlp_loss_grad and dct_mlp_adam
     float* grad = reinterpret_cast<float*>(static_cast<char*>(workspace) + dct_mlp_workspace_bytes(batch));
     for (int b0 = 0, k = 0; b0 < n; b0 += batch, ++k) {
         const int cnt = n - b0 < batch ? n - b0 : batch;
-        cudaError_t e = launch_train_step<true>(net, feats, labels, order + b0, cnt, grad, loss_out + k, workspace,
-                                                next_adam_step(net, lr, 0.9f, 0.999f, 1e-8f), (cudaStream_t)stream);
+        cudaError_t e = launch_loss_grad(net, feats, labels, order + b0, cnt, grad, loss_out + k, workspace, st_);
         if (e != cudaSuccess) return cuda_fail(e, "training step launch");
+        if ((st = dct_mlp_adam(net, grad, lr, 0.9f, 0.999f, 1e-8f, stream)) != DCT_OK) return st;
     }
     return DCT_OK;
 }

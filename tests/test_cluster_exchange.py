@@ -18,7 +18,8 @@ def test_no_kernel_names(word):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("steps,batch,last", [(64, 64, 64), (65, 64, 1), (131, 64, 7), (66, 300, 257), (65, 1024, 700)])
+@pytest.mark.parametrize("steps,batch,last", [(64, 64, 64), (65, 64, 1), (131, 64, 7), (66, 300, 257), (65, 1024, 700),
+                                              (131, 1, 1), (70, 33, 5), (3, 5000, 4999)])
 def test_epoch_of_several_launches(cuda_ok, steps, batch, last):
     import torch
 
