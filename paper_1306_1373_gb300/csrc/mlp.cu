@@ -36,67 +36,98 @@ __device__ __forceinline__ float act(float h, int bf16) {
     return bf16 ? __bfloat162float(__float2bfloat16_rn(h)) : h;
 }
 
-// Inference, one warp per sample: lane l owns hidden units l and l + 32 of both
-// layers, every sum over its inputs in ascending order (the inputs a lane does
-// not hold come by shuffle).  W1 and W2 are staged transposed with rows padded
-// to 65 floats, as in k_mlp_delta.  One thread per sample took 219 us for the
-// 48 frames of a small rate-control call (a serial walk over 9,409 parameters
-// in global memory); this takes 10 us.
-constexpr int kFwdRows = 8;                    // samples (warps) per CTA
+// Inference, ROWS samples to a warp: lane l owns hidden units l and l + 32 of
+// both layers, every sum over its inputs in ascending order (the inputs a lane
+// does not hold come by shuffle).  W1 and W2 are staged transposed with rows
+// padded to 65 floats, as in k_mlp_delta.  One thread per sample took 219 us for
+// the 48 frames of a small rate-control call (a serial walk over 9,409
+// parameters in global memory); one sample a warp takes 13 us.  That is bound
+// by the shared-memory pipe, which also moves the shuffles; four samples a warp
+// read a weight once for four: 100,000 samples 144 us against 213, 1,000,000
+// 1346 against 2000 (1905 with a thread per sample).
+constexpr int kFwdWarps = 8;                   // warps per CTA
 constexpr int kTStride = kHid + 1;             // padded row of a transposed weight matrix
 
-__global__ void __launch_bounds__(kFwdRows * 32)
+template <int ROWS>
+__global__ void __launch_bounds__(kFwdWarps * 32)
 k_mlp_forward(const float* __restrict__ P, const float* __restrict__ feats, const float* __restrict__ mean,
               const float* __restrict__ stdv, int bf16, int n, float* __restrict__ y_out, int* __restrict__ q_out) {
     __shared__ float w1t[kIn * kTStride];       // w1t[i * 65 + j] = W1[j][i]
     __shared__ float w2t[kHid * kTStride];
 #pragma unroll 8
-    for (int e = threadIdx.x; e < kHid * kIn; e += kFwdRows * 32) w1t[(e % kIn) * kTStride + e / kIn] = P[oW1 + e];
+    for (int e = threadIdx.x; e < kHid * kIn; e += kFwdWarps * 32) w1t[(e % kIn) * kTStride + e / kIn] = P[oW1 + e];
 #pragma unroll 8
-    for (int e = threadIdx.x; e < kHid * kHid; e += kFwdRows * 32) w2t[(e % kHid) * kTStride + e / kHid] = P[oW2 + e];
+    for (int e = threadIdx.x; e < kHid * kHid; e += kFwdWarps * 32) w2t[(e % kHid) * kTStride + e / kHid] = P[oW2 + e];
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    for (int s = blockIdx.x * kFwdRows + (threadIdx.x >> 5); s < n; s += gridDim.x * kFwdRows) {   // warp-uniform
-        const float* x = feats + (size_t)s * kIn;
-        float xn[3];
+    const long long step = (long long)gridDim.x * kFwdWarps * ROWS;
+    for (long long s = ((long long)blockIdx.x * kFwdWarps + (threadIdx.x >> 5)) * ROWS; s < n; s += step) {   // warp-uniform
+        float xn[ROWS][3];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const int i = lane + 32 * k;
-            xn[k] = i < kIn ? (x[i] - mean[i]) / stdv[i] : 0.0f;
+        for (int r = 0; r < ROWS; ++r) {
+            const float* x = feats + (size_t)(ROWS == 1 || s + r < n ? s + r : s) * kIn;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const int i = lane + 32 * k;
+                xn[r][k] = i < kIn ? (x[i] - mean[i]) / stdv[i] : 0.0f;
+            }
         }
-        float a[2], h[2];
+        float a[ROWS][2], h[ROWS][2], z[ROWS];
 #pragma unroll
-        for (int k = 0; k < 2; ++k) a[k] = P[oB1 + lane + 32 * k];
+        for (int r = 0; r < ROWS; ++r) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) a[r][k] = P[oB1 + lane + 32 * k];
+        }
 #pragma unroll
         for (int i = 0; i < kIn; ++i) {
-            const float v = __shfl_sync(0xffffffffu, xn[i >> 5], i & 31);
+            const float w[2] = {w1t[i * kTStride + lane], w1t[i * kTStride + lane + 32]};
 #pragma unroll
-            for (int k = 0; k < 2; ++k) a[k] = fmaf(w1t[i * kTStride + lane + 32 * k], v, a[k]);
+            for (int r = 0; r < ROWS; ++r) {
+                const float v = __shfl_sync(0xffffffffu, xn[r][i >> 5], i & 31);
+#pragma unroll
+                for (int k = 0; k < 2; ++k) a[r][k] = fmaf(w[k], v, a[r][k]);
+            }
         }
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            h[k] = act(gelu(a[k]), bf16);
-            a[k] = P[oB2 + lane + 32 * k];
+        for (int r = 0; r < ROWS; ++r) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                h[r][k] = act(gelu(a[r][k]), bf16);
+                a[r][k] = P[oB2 + lane + 32 * k];
+            }
         }
 #pragma unroll
         for (int i = 0; i < kHid; ++i) {
-            const float v = __shfl_sync(0xffffffffu, h[i >> 5], i & 31);
+            const float w[2] = {w2t[i * kTStride + lane], w2t[i * kTStride + lane + 32]};
 #pragma unroll
-            for (int k = 0; k < 2; ++k) a[k] = fmaf(w2t[i * kTStride + lane + 32 * k], v, a[k]);
+            for (int r = 0; r < ROWS; ++r) {
+                const float v = __shfl_sync(0xffffffffu, h[r][i >> 5], i & 31);
+#pragma unroll
+                for (int k = 0; k < 2; ++k) a[r][k] = fmaf(w[k], v, a[r][k]);
+            }
         }
 #pragma unroll
-        for (int k = 0; k < 2; ++k) h[k] = act(gelu(a[k]), bf16);
-        const float w3[2] = {P[oW3 + lane], P[oW3 + lane + 32]};
-        float z = P[oB3];
+        for (int r = 0; r < ROWS; ++r) {
 #pragma unroll
-        for (int j = 0; j < kHid; ++j)
-            z = fmaf(__shfl_sync(0xffffffffu, w3[j >> 5], j & 31), __shfl_sync(0xffffffffu, h[j >> 5], j & 31), z);
-        const float y = 1.0f / (1.0f + expf(-z));
-        if (lane == 0) {
-            if (y_out) y_out[s] = y;
-            if (q_out) {
-                const float q = rintf(1.0f + 99.0f * y);
-                q_out[s] = (int)fminf(100.0f, fmaxf(1.0f, q));
+            for (int k = 0; k < 2; ++k) h[r][k] = act(gelu(a[r][k]), bf16);
+            z[r] = P[oB3];
+        }
+        const float w3[2] = {P[oW3 + lane], P[oW3 + lane + 32]};
+#pragma unroll
+        for (int j = 0; j < kHid; ++j) {
+            const float w = __shfl_sync(0xffffffffu, w3[j >> 5], j & 31);
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) z[r] = fmaf(w, __shfl_sync(0xffffffffu, h[r][j >> 5], j & 31), z[r]);
+        }
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+            const float y = 1.0f / (1.0f + expf(-z[r]));
+            if (lane == 0 && (ROWS == 1 || s + r < n)) {
+                if (y_out) y_out[s + r] = y;
+                if (q_out) {
+                    const float q = rintf(1.0f + 99.0f * y);
+                    q_out[s + r] = (int)fminf(100.0f, fmaxf(1.0f, q));
+                }
             }
         }
     }
@@ -894,9 +925,13 @@ cudaError_t launch_features(const unsigned long long* stats, const int* w, const
 }
 
 cudaError_t launch_mlp_forward(const dct_mlp* net, const float* feats, int n, float* y, int* q, cudaStream_t s) {
-    const int ctas = (n + kFwdRows - 1) / kFwdRows;
-    k_mlp_forward<<<ctas < 1024 ? ctas : 1024, kFwdRows * 32, 0, s>>>(net->params, feats, net->feat_mean, net->feat_std, net->act_bf16, n,
-                                               y, q);
+    // four samples a warp as soon as that leaves every SM a CTA (8,000 samples 23
+    // us against 27, 4,000 19 either way, 1,000 19 against 13)
+    const bool four = n >= 4 * kFwdWarps * 152;
+    const auto kernel = four ? k_mlp_forward<4> : k_mlp_forward<1>;
+    const long long rows = (four ? 4 : 1) * kFwdWarps, ctas = (n + rows - 1) / rows;
+    kernel<<<ctas < 1024 ? (int)ctas : 1024, kFwdWarps * 32, 0, s>>>(net->params, feats, net->feat_mean, net->feat_std,
+                                                                   net->act_bf16, n, y, q);
     return cudaGetLastError();
 }
 
