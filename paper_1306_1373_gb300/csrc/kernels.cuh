@@ -103,12 +103,16 @@ enum : unsigned {
 // u and v are both 0 or 4 (g_u g_v = 1, M = rint(2^25 / Q) a high power of two
 // for Q = 1, 2, 4, ...); there the multiplier is the next float above
 // M * 2^-32, which lifts the exact halves over the half and moves no other
-// product across one (a test runs every reachable M over every |Y|).
+// product across one (tests run every M at kN = 6, and those of 15 steps at kN = 4
+// and 5, over every |Y|; that no half occurs elsewhere, at every step and kN).
 // M must fit a float's 24 bits: only M > 2^24 (Q = 1, and Q = 2 at the
 // smallest gains; quality 93 and up) may not, and tables with such an entry
 // take the integer form (Mf[0] = 0).  The integer form costs a 64-bit multiply,
 // which issues at 1/8 of the FMA rate (measured: 16 against 128 per clock per
-// SM); this one costs half an issue slot.
+// SM), and the conversions around it; this one costs half an issue slot.  Fused
+// graph, 60 M samples: 106.5 us at quality 75, 112.7 at 95 (114.8 with the
+// result's conversion in an addition of its own; 111 with integer arithmetic
+// throughout, which takes 111 at quality 75 too).
 constexpr float kMagic = 12582912.0f;               // 1.5 * 2^23
 constexpr int kMagicBits = 0x4B400000;              // its bits: bits(kMagic + q) = kMagicBits + q
 __host__ __device__ constexpr bool tie_entry(int u, int v) { return (u & 3) == 0 && (v & 3) == 0; }
@@ -132,11 +136,12 @@ __host__ __device__ inline bool quant_multiplier(uint32_t m, float& out) {
 template <bool FLT, int U, int V>
 __device__ __forceinline__ float quant_code(float y, float mf, const uint32_t* M) {
     if constexpr (FLT) return __fmaf_rn(y, mf, kMagic);
-    // high word of Y M + 2^31, with - [Y < 0] where halves can occur (M < 2^26)
+    // high word of Y M + 2^31, with - [Y < 0] where halves can occur (M < 2^26);
+    // kMagicBits comes with the addend (the sum stays below 2^63)
     const int yi = __float_as_int(__fadd_rn(y, kMagic)) - kMagicBits;
-    long long p = (long long)yi * (long long)(int)M[U * 8 + V] + 0x80000000ll;
+    long long p = (long long)yi * (long long)(int)M[U * 8 + V] + (((long long)kMagicBits << 32) + 0x80000000ll);
     if (tie_entry(U, V)) p += (long long)(yi >> 31);
-    return __int_as_float((int)(p >> 32) + kMagicBits);
+    return __int_as_float((int)(p >> 32));
 }
 
 // An own code kMagic + q, dequantised: G = q (Q W) as the integer kMagicBits +
