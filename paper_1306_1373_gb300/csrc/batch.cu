@@ -165,7 +165,8 @@ __global__ void __launch_bounds__(256, DCTGB_MINB) k_batch(const __grid_constant
 // straight from global memory (the 32 resident warps per SM hide the latency
 // that the one-lane kernel hides with cp.async prefetch).  Claimed tiles only
 // increase, so a warp still meets each item's tiles in order.  CHUNK > 1
-// spares the counter on large batches (many tiles per warp).
+// spares the counter on large batches (many tiles per warp); CHUNK 0 hands out
+// half tiles (units of 16 blocks) where there are fewer tiles than warps.
 template <unsigned MODE, int CHUNK>
 __global__ void __launch_bounds__(256, DCTGB_PAIR_MINB) k_batch_pair(const __grid_constant__ BatchArgs args) {
     extern __shared__ __align__(16) uint8_t smem[];
@@ -178,29 +179,33 @@ __global__ void __launch_bounds__(256, DCTGB_PAIR_MINB) k_batch_pair(const __gri
     PlaneArg& P = *reinterpret_cast<PlaneArg*>(base + kTabBytes);
     uint8_t* xb = base + kTabBytes + kDescBytes;
 
+    constexpr bool kHalves = CHUNK == 0;
+    constexpr int kClaim = kHalves ? 1 : CHUNK;
     const bool claim = args.next_tile != nullptr;
-    int tile = 0, limit = 0;
+    const int units = kHalves ? 2 * args.ntiles : args.ntiles;
+    int unit = 0, limit = 0;
     if (!claim) {
         const long long total_warps = (long long)gridDim.x * warps_per_cta;
         const long long gw = (long long)blockIdx.x * warps_per_cta + warp;
-        tile = (int)((gw * args.ntiles) / total_warps);
-        limit = (int)(((gw + 1) * args.ntiles) / total_warps);
+        unit = (int)((gw * units) / total_warps);
+        limit = (int)(((gw + 1) * units) / total_warps);
     }
 
     int cur = -1;
     int item_end = 0;
     unsigned long long* item_sse = nullptr;
     unsigned long long sse = 0ull;
-    for (;; ++tile) {
-        if (tile >= limit) {
+    for (;; ++unit) {
+        if (unit >= limit) {
             if (!claim) break;
             int t = 0;
-            if (lane == 0) t = (int)atomicAdd(args.next_tile, (unsigned)CHUNK);
+            if (lane == 0) t = (int)atomicAdd(args.next_tile, (unsigned)kClaim);
             t = __shfl_sync(0xffffffffu, t, 0);
-            if (t >= args.ntiles) break;
-            tile = t;
-            limit = CHUNK == 1 ? t + 1 : min(t + CHUNK, args.ntiles);
+            if (t >= units) break;
+            unit = t;
+            limit = kClaim == 1 ? t + 1 : min(t + kClaim, units);
         }
+        const int tile = kHalves ? unit >> 1 : unit, first = kHalves ? unit & 1 : 0;
         if (cur < 0 || tile >= item_end) {
             __syncwarp();
             if ((MODE & kSse) && cur >= 0 && lane == 0 && sse) atomicAdd(item_sse, sse);
@@ -214,7 +219,8 @@ __global__ void __launch_bounds__(256, DCTGB_PAIR_MINB) k_batch_pair(const __gri
             copy_table<kTabBytes>(base, args.tabs + __ldg(&gi->table), pair_tab_first(MODE), lane);
             __syncwarp();
         }
-        sse += process_tile_pair<MODE>(P, pair_tabs<MODE>(base), tile - P.tile_begin, lane, xb);
+        sse += process_tile_pair<MODE>(P, pair_tabs<MODE>(base), tile - P.tile_begin, lane, xb, first,
+                                       kHalves ? first + 1 : 2);
     }
     if ((MODE & kSse) && cur >= 0 && lane == 0 && sse) atomicAdd(item_sse, sse);
 }
@@ -260,15 +266,19 @@ static KernelPtr pair_kernel_c(unsigned mode) {
     }
 }
 
-// Tiles a warp claims at a time: four once a launch has at least 16 tiles
-// per warp (the 512-image batch, about 60 per warp: 602 vs 577 GPix/s
-// measured), else one (the benchmark planes, about 8 per warp), so the last
-// claims still spread over all warps.
+// What a warp of a two-lane kernel claims at a time (W: resident warps).  Four
+// tiles once a launch has at least 16 per warp (the 512-image batch, about 60
+// per warp: 602 vs 577 GPix/s measured), else one (the benchmark planes, about
+// 8 per warp), so the last claims still spread over all warps.  Half a tile
+// while there are fewer tiles than warps: each warp then has one claim's latency
+// (fused graph at the default shape, us, halves against tiles: 1 M samples 12.1 /
+// 15.0, 4 M (0.5 tiles per warp) 19.2 / 20.6, 6 M (0.8) 21.7 / 23.9; beyond, the
+// last round of claims costs more: 10 M (1.3) 31.1 / 29.1, 14 M (1.9) 37.9 / 37.1).
 constexpr int kClaimChunk = 4;
 constexpr int kChunkTilesPerWarp = 16;
 
-static KernelPtr pair_kernel(unsigned mode, bool chunked = false) {
-    return chunked ? pair_kernel_c<kClaimChunk>(mode) : pair_kernel_c<1>(mode);
+static KernelPtr pair_kernel(unsigned mode, int chunk = 1) {
+    return chunk == 0 ? pair_kernel_c<0>(mode) : chunk == 1 ? pair_kernel_c<1>(mode) : pair_kernel_c<kClaimChunk>(mode);
 }
 
 // Two lanes per block when the shape asks for it and the mode has a two-lane
@@ -301,8 +311,8 @@ static KernelPtr one_lane_kernel(unsigned mode) {
     }
 }
 
-static KernelPtr batch_kernel(unsigned mode, const dct_launch_shape& sh, bool chunked = false) {
-    return use_pair(mode, sh) ? pair_kernel(mode, chunked) : one_lane_kernel(mode);
+static KernelPtr batch_kernel(unsigned mode, const dct_launch_shape& sh, int chunk = 1) {
+    return use_pair(mode, sh) ? pair_kernel(mode, chunk) : one_lane_kernel(mode);
 }
 
 struct BatchState {
@@ -371,20 +381,23 @@ static size_t batch_smem(int threads, unsigned mode, const dct_launch_shape& sh)
     return (size_t)(threads / 32) * (use_pair(mode, sh) ? pair_warp_smem_bytes(mode) : warp_smem_bytes(mode));
 }
 
-static int batch_grid(const dct_plan_s* plan, unsigned mode, const dct_launch_shape& sh, int ntiles) {
-    const int threads = sh.threads_per_cta;
-    int per_sm = sh.ctas_per_sm;
-    if (per_sm <= 0) {
-        int occ = 1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, batch_kernel(mode, sh), threads,
-                                                          batch_smem(threads, mode, sh)) !=
-                cudaSuccess || occ < 1)
-            occ = 1;
-        per_sm = occ;
-    }
-    const int warps = threads / 32;
-    const int need = std::max(1, (ntiles + warps - 1) / warps);
-    return std::min(need, plan->num_sms * per_sm);
+struct BatchGrid {
+    int ctas, chunk;              // chunk: what a two-lane kernel's warps claim (pair_kernel)
+};
+
+static BatchGrid batch_grid(const dct_plan_s* plan, unsigned mode, const dct_launch_shape& sh, int ntiles) {
+    const int threads = sh.threads_per_cta, warps = threads / 32;
+    int occ = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, batch_kernel(mode, sh), threads,
+                                                      batch_smem(threads, mode, sh)) != cudaSuccess || occ < 1)
+        occ = 1;
+    const int per_sm = sh.ctas_per_sm > 0 ? sh.ctas_per_sm : occ;
+    BatchGrid g{0, 1};
+    if (use_pair(mode, sh) && ntiles < plan->num_sms * std::min(per_sm, occ) * warps) g.chunk = 0;
+    const int units = g.chunk == 0 ? 2 * ntiles : ntiles;
+    g.ctas = std::min(std::max(1, (units + warps - 1) / warps), plan->num_sms * per_sm);
+    if (use_pair(mode, sh) && (long long)ntiles >= (long long)kChunkTilesPerWarp * g.ctas * warps) g.chunk = kClaimChunk;
+    return g;
 }
 
 // Records [init, kernel(s)] on the capture stream and instantiates the graph.
@@ -412,13 +425,12 @@ static dct_status capture(dct_plan_t plan, const dct_launch_shape& sh) {
     a.nitems = b->n;
     a.ntiles = b->ntiles;
     for (int k = 0; k < b->nkernels; ++k) {
-        const int grid = batch_grid(plan, b->modes[k], sh, b->ntiles);
-        const bool chunked = (long long)b->ntiles >= (long long)kChunkTilesPerWarp * grid * (sh.threads_per_cta / 32);
-        KernelPtr kp = batch_kernel(b->modes[k], sh, chunked);
+        const BatchGrid grid = batch_grid(plan, b->modes[k], sh, b->ntiles);
+        KernelPtr kp = batch_kernel(b->modes[k], sh, grid.chunk);
         const size_t smem = batch_smem(sh.threads_per_cta, b->modes[k], sh);
         a.next_tile = use_pair(b->modes[k], sh) ? b->d_counters + k : nullptr;
         cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        kp<<<grid, sh.threads_per_cta, smem, s>>>(a);
+        kp<<<grid.ctas, sh.threads_per_cta, smem, s>>>(a);
     }
     cudaGraph_t graph = nullptr;
     cudaError_t e2 = cudaGetLastError();
@@ -446,10 +458,8 @@ cudaError_t batch_launch(unsigned mode, const PlaneArg* items, const int32_t* ti
     dct_launch_shape sh = plan->shape;
     if (!valid_shape(sh)) sh = default_shape();
     if (!batch_kernel(mode, sh)) return cudaErrorInvalidValue;
-    const int grid = batch_grid(plan, mode, sh, ntiles);
-    const bool claim = tile_counter != nullptr && use_pair(mode, sh);
-    const bool chunked = claim && (long long)ntiles >= (long long)kChunkTilesPerWarp * grid * (sh.threads_per_cta / 32);
-    KernelPtr kp = batch_kernel(mode, sh, chunked);
+    const BatchGrid grid = batch_grid(plan, mode, sh, ntiles);
+    KernelPtr kp = batch_kernel(mode, sh, grid.chunk);
     const size_t smem = batch_smem(sh.threads_per_cta, mode, sh);
     cudaError_t e = cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -459,8 +469,8 @@ cudaError_t batch_launch(unsigned mode, const PlaneArg* items, const int32_t* ti
     a.tabs = tabs;
     a.nitems = nitems;
     a.ntiles = ntiles;
-    a.next_tile = claim ? tile_counter : nullptr;
-    kp<<<grid, sh.threads_per_cta, smem, s>>>(a);
+    a.next_tile = use_pair(mode, sh) ? tile_counter : nullptr;
+    kp<<<grid.ctas, sh.threads_per_cta, smem, s>>>(a);
     return cudaGetLastError();
 }
 
