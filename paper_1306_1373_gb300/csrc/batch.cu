@@ -24,7 +24,8 @@ namespace dctgb {
 struct BatchArgs {
     const PlaneArg* items;      // device work list
     const int32_t* tile_begin;  // nitems + 1 prefix offsets
-    const QuantSet* tabs;       // unique tables
+    const uint8_t* tabs;        // unique tables: byte b of set k is at k * tab_stride + b
+    int64_t tab_stride;         // (sizeof(QuantSet), or less where only a part is kept)
     int32_t nitems;
     int32_t ntiles;
     // Two-lane kernels: when set, warps claim tiles from this counter (zero on
@@ -68,9 +69,9 @@ __device__ __forceinline__ void flush_stats(const unsigned long long* wst, unsig
 // in turn: fused graph of 2 M samples, one lane per block, one tile a warp, 14.5 us
 // against 15.8.)
 template <int BYTES>
-__device__ __forceinline__ void copy_table(uint8_t* dst, const QuantSet* set, int first, int lane) {
+__device__ __forceinline__ void copy_table(uint8_t* dst, const BatchArgs& args, int set, int first, int lane) {
     constexpr int kLoads = (BYTES / 16 + 31) / 32;
-    const uint4* s = reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(set) + first);
+    const uint4* s = reinterpret_cast<const uint4*>(args.tabs + set * args.tab_stride + first);
     uint4 v[kLoads];
 #pragma unroll
     for (int k = 0; k < kLoads; ++k)
@@ -125,7 +126,7 @@ __global__ void __launch_bounds__(256, DCTGB_MINB) k_batch(const __grid_constant
             if (lane < (int)(sizeof(PlaneArg) / 4))
                 reinterpret_cast<uint32_t*>(&P)[lane] = __ldg(reinterpret_cast<const uint32_t*>(gi) + lane);
             copy_table<pair_tab_bytes(MODE)>(reinterpret_cast<uint8_t*>(T) + pair_tab_first(MODE),
-                                             args.tabs + __ldg(&gi->table), pair_tab_first(MODE), lane);
+                                             args, __ldg(&gi->table), pair_tab_first(MODE), lane);
             __syncwarp();
             pf_valid = false;
         }
@@ -216,7 +217,7 @@ __global__ void __launch_bounds__(256, DCTGB_PAIR_MINB) k_batch_pair(const __gri
             item_sse = gi->sse;
             if (lane < (int)(sizeof(PlaneArg) / 4))
                 reinterpret_cast<uint32_t*>(&P)[lane] = __ldg(reinterpret_cast<const uint32_t*>(gi) + lane);
-            copy_table<kTabBytes>(base, args.tabs + __ldg(&gi->table), pair_tab_first(MODE), lane);
+            copy_table<kTabBytes>(base, args, __ldg(&gi->table), pair_tab_first(MODE), lane);
             __syncwarp();
         }
         sse += process_tile_pair<MODE>(P, pair_tabs<MODE>(base), tile - P.tile_begin, lane, xb, first,
@@ -421,7 +422,8 @@ static dct_status capture(dct_plan_t plan, const dct_launch_shape& sh) {
     BatchArgs a;
     a.items = b->d_items;
     a.tile_begin = b->d_tile_begin;
-    a.tabs = b->d_tabs;
+    a.tabs = reinterpret_cast<const uint8_t*>(b->d_tabs);
+    a.tab_stride = sizeof(QuantSet);
     a.nitems = b->n;
     a.ntiles = b->ntiles;
     for (int k = 0; k < b->nkernels; ++k) {
@@ -453,8 +455,9 @@ static bool valid_shape(const dct_launch_shape& sh) {
            sh.lanes_per_block >= 0 && sh.lanes_per_block <= 2;
 }
 
-cudaError_t batch_launch(unsigned mode, const PlaneArg* items, const int32_t* tile_begin, const QuantSet* tabs,
-                         int nitems, int ntiles, const dct_plan_s* plan, cudaStream_t s, unsigned int* tile_counter) {
+cudaError_t batch_launch(unsigned mode, const PlaneArg* items, const int32_t* tile_begin, const void* tabs,
+                         int nitems, int ntiles, const dct_plan_s* plan, cudaStream_t s, unsigned int* tile_counter,
+                         size_t tab_stride) {
     dct_launch_shape sh = plan->shape;
     if (!valid_shape(sh)) sh = default_shape();
     if (!batch_kernel(mode, sh)) return cudaErrorInvalidValue;
@@ -466,7 +469,8 @@ cudaError_t batch_launch(unsigned mode, const PlaneArg* items, const int32_t* ti
     BatchArgs a;
     a.items = items;
     a.tile_begin = tile_begin;
-    a.tabs = tabs;
+    a.tabs = static_cast<const uint8_t*>(tabs);
+    a.tab_stride = (int64_t)tab_stride;
     a.nitems = nitems;
     a.ntiles = ntiles;
     a.next_tile = use_pair(mode, sh) ? tile_counter : nullptr;

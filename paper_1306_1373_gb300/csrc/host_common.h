@@ -69,10 +69,12 @@ void batch_release(dct_plan_t plan);
 // Launches the batched persistent kernel of `mode` over a device work list
 // (no graph), with the plan's launch shape (batch.cu).  With tile_counter (a
 // device word the caller has zeroed on `s` before the launch) a two-lane
-// kernel claims its tiles from it; without, warps take fixed ranges.
-cudaError_t batch_launch(unsigned mode, const PlaneArg* items, const int32_t* tile_begin, const QuantSet* tabs,
+// kernel claims its tiles from it; without, warps take fixed ranges.  Byte b of
+// table set k is at tabs + k * tab_stride + b; only the mode's part (pair_tab_first,
+// pair_tab_bytes) is read.
+cudaError_t batch_launch(unsigned mode, const PlaneArg* items, const int32_t* tile_begin, const void* tabs,
                          int nitems, int ntiles, const dct_plan_s* plan, cudaStream_t s,
-                         unsigned int* tile_counter = nullptr);
+                         unsigned int* tile_counter = nullptr, size_t tab_stride = sizeof(QuantSet));
 
 // Frees the plan's rate-control workspace (ratecontrol.cu).
 void rc_release(dct_plan_t plan);

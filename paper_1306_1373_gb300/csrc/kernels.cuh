@@ -36,13 +36,16 @@ constexpr int kPixBytes = kTileBlocks * 64;       // one tile of uint8 samples
 // Per-plane quantiser / dequantiser tables (natural order u*8+v).
 // The float entries drive the kernels that quantise on the FMA pipes (see
 // quant_code and dequant_bits).
+// In the order of the parts that the batched kernels copy: the inverse of own
+// codes reads QWi, the forward pass M and Mf, the fused one M to QWc, the inverse
+// of any codes Q and W, and a two-pass batch QWi to Mf.
 struct QuantSet {
+    int32_t QWi[64];  // Q * W
     uint32_t M[64];   // rint(2^32 / (8 * 2^P * g_u g_v Q))
     float Mf[64];     // M * 2^-32, with the tie rule of quant_multiplier;
                       // Mf[0] = 0 when some M does not fit 24 bits
     float QW[64];     // Q * W
     float QWc[64];    // kMagic * (1 - Q * W)
-    int32_t QWi[64];  // Q * W
     int32_t Q[64];    // 1..255
     int32_t W[64];    // rint(2^R / (g_u g_v))
 };

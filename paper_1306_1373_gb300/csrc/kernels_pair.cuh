@@ -41,15 +41,15 @@ constexpr int kXRowHalf = 144;                    // offset of rows 4..7 in a sl
 constexpr int kXBytes = kPairBlocks * kXSlot;     // per warp
 constexpr int kParkBytes = 32 * 32;               // each lane's 32 samples, kept for the SSE
 
-// The part of a QuantSet that a mode reads: [M, Mf, QW, QWc] forward and fused,
-// [QWi] for the inverse of own codes, [Q, W] for the inverse of any codes.
+// The part of a QuantSet that a mode reads: [M, Mf, QW, QWc] fused, [M, Mf]
+// forward, [QWi] for the inverse of own codes, [Q, W] for the inverse of any.
 // Batched warps keep only that part, so that 32 warps' slots fit an SM.
 __host__ __device__ constexpr int pair_tab_first(unsigned mode) {
     return (mode & kLoadPix) ? (int)offsetof(QuantSet, M)
                              : (mode & kOwnCodes) ? (int)offsetof(QuantSet, QWi) : (int)offsetof(QuantSet, Q);
 }
 __host__ __device__ constexpr int pair_tab_bytes(unsigned mode) {
-    return (mode & kLoadPix) ? 4 * 256 : (mode & kOwnCodes) ? 256 : 2 * 256;
+    return (mode & kLoadPix) ? ((mode & kInverse) ? 4 : 2) * 256 : (mode & kOwnCodes) ? 256 : 2 * 256;
 }
 struct PairTabs {
     const uint32_t* M;

@@ -24,18 +24,30 @@
 #include <cstring>
 
 #include "host_common.h"
+#include "kernels_pair.cuh"
 
 namespace dctgb {
 
 // Largest batch the static work list holds.
 constexpr int kNoAllocMaxItems = 64;
 
+// Of a table set the list holds the part that the operation's kernels read: one
+// part, or for the two-pass operation the neighbouring parts of its two kernels.
+constexpr unsigned kTwoPassFwd = kLoadPix | kStoreCoef, kTwoPassInv = kLoadCoef | kInverse | kOwnCodes;
+constexpr int kNoAllocTabBytes = 1024;
+static_assert(pair_tab_bytes(kLoadPix | kInverse) <= kNoAllocTabBytes && pair_tab_bytes(kLoadCoef | kInverse) <= kNoAllocTabBytes,
+              "the parts fit");
+static_assert(pair_tab_first(kTwoPassInv) < pair_tab_first(kTwoPassFwd) &&
+                  pair_tab_first(kTwoPassFwd) + pair_tab_bytes(kTwoPassFwd) <= pair_tab_first(kTwoPassInv) + kNoAllocTabBytes,
+              "the two-pass parts fit together");
+
 struct NoAllocList {
     PlaneArg items[kNoAllocMaxItems];
     int32_t tile_begin[kNoAllocMaxItems + 1];
     int32_t pad[(256 - ((kNoAllocMaxItems + 1) * 4) % 256) / 4];
-    QuantSet tabs[kNoAllocMaxItems];
+    uint8_t tabs[kNoAllocMaxItems][kNoAllocTabBytes];
 };
+static_assert(offsetof(NoAllocList, tabs) % 16 == 0 && sizeof(NoAllocList) <= 72 * 1024, "the size that dctgb.h states");
 
 // The scratch: one work list shared by every call on a device.
 static __device__ __align__(256) NoAllocList g_noalloc_list;
@@ -184,13 +196,16 @@ extern "C" dct_status dct_batch_run_noalloc(const dct_batch_item* items, int n, 
     if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
     plan.device = dev;
 
-    // Pass 2: upload the distinct tables from one stack buffer each, then
-    // the descriptors (pageable copies: cudaMemcpyAsync has read them when
+    // Pass 2: upload the parts of the distinct tables from one stack buffer,
+    // then the descriptors (pageable copies: cudaMemcpyAsync has read them when
     // it returns).
+    const int first = pair_tab_first(mode);               // of the two parts of a two-pass operation the inverse one is first
+    const int bytes = two ? pair_tab_first(kTwoPassFwd) + pair_tab_bytes(kTwoPassFwd) - first : pair_tab_bytes(mode);
+    const void* const tabs = reinterpret_cast<const void*>(reinterpret_cast<uintptr_t>(dlist->tabs) - first);
     for (int k = 0; k < ntabs; ++k) {
         const dct_batch_item& it = items[tab_item[k]];
         build_tables(it.quality, it.qtab_host, 64, it.chroma, tab);
-        e = cudaMemcpyAsync(dlist->tabs + k, &tab, sizeof(QuantSet), cudaMemcpyHostToDevice, s);
+        e = cudaMemcpyAsync(dlist->tabs[k], reinterpret_cast<const uint8_t*>(&tab) + first, bytes, cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) return cuda_fail(e, "table upload");
     }
     e = cudaMemcpyAsync(dlist->items, h.items, sizeof(PlaneArg) * n, cudaMemcpyHostToDevice, s);
@@ -202,10 +217,10 @@ extern "C" dct_status dct_batch_run_noalloc(const dct_batch_item* items, int n, 
         if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "SSE clear launch");
     }
     if (two) {
-        e = batch_launch(kLoadPix | kStoreCoef, dlist->items, dlist->tile_begin, dlist->tabs, n, cursor, &plan, s);
+        e = batch_launch(kTwoPassFwd, dlist->items, dlist->tile_begin, tabs, n, cursor, &plan, s, nullptr, kNoAllocTabBytes);
         if (e != cudaSuccess) return cuda_fail(e, "forward launch");
     }
-    e = batch_launch(mode, dlist->items, dlist->tile_begin, dlist->tabs, n, cursor, &plan, s);
+    e = batch_launch(mode, dlist->items, dlist->tile_begin, tabs, n, cursor, &plan, s, nullptr, kNoAllocTabBytes);
     if (e != cudaSuccess) return cuda_fail(e, "batch launch");
     return DCT_OK;
 }
