@@ -25,7 +25,7 @@ struct BatchArgs {
     const PlaneArg* items;      // device work list
     const int32_t* tile_begin;  // nitems + 1 prefix offsets
     const uint8_t* tabs;        // unique tables: byte b of set k is at k * tab_stride + b
-    int64_t tab_stride;         // (sizeof(QuantSet), or less where only a part is kept)
+    int32_t tab_stride;         // (sizeof(QuantSet), or less where only a part is kept)
     int32_t nitems;
     int32_t ntiles;
     // Two-lane kernels: when set, warps claim tiles from this counter (zero on
@@ -71,7 +71,7 @@ __device__ __forceinline__ void flush_stats(const unsigned long long* wst, unsig
 template <int BYTES>
 __device__ __forceinline__ void copy_table(uint8_t* dst, const BatchArgs& args, int set, int first, int lane) {
     constexpr int kLoads = (BYTES / 16 + 31) / 32;
-    const uint4* s = reinterpret_cast<const uint4*>(args.tabs + set * args.tab_stride + first);
+    const uint4* s = reinterpret_cast<const uint4*>(args.tabs + (unsigned)(set * args.tab_stride) + first);
     uint4 v[kLoads];
 #pragma unroll
     for (int k = 0; k < kLoads; ++k)
@@ -470,7 +470,7 @@ cudaError_t batch_launch(unsigned mode, const PlaneArg* items, const int32_t* ti
     a.items = items;
     a.tile_begin = tile_begin;
     a.tabs = static_cast<const uint8_t*>(tabs);
-    a.tab_stride = (int64_t)tab_stride;
+    a.tab_stride = (int32_t)tab_stride;
     a.nitems = nitems;
     a.ntiles = ntiles;
     a.next_tile = use_pair(mode, sh) ? tile_counter : nullptr;
