@@ -123,9 +123,10 @@ constexpr bool kTrOffsets = kN <= 6;
 // Starting offsets, lifted step by step: the solution of steps 1..i-1 is known
 // modulo 2^(1 + .. + i-1), and step i picks its next i bits of each.
 constexpr FltBias tr_start(unsigned mask) {
+    if (!kTrOffsets) return {0, 0};
     long long ka = 0, kb = 0;
     int bits = 0;
-    for (int i = 1; i <= kN && kTrOffsets; ++i) {
+    for (int i = 1; i <= kN; ++i) {
         bool found = false;
         for (long long x = 0; x < (1LL << i) && !found; ++x)
             for (long long y = 0; y < (1LL << i) && !found; ++y)
