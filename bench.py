@@ -1143,7 +1143,7 @@ def main():
         sets[1]["plan"].close()
 
     # ---- roofline of the dominant kernel.  The path is bound by integer
-    # instruction issue (ncu: issue slots ~80% busy, DRAM ~25%), so the
+    # instruction issue (ncu: issue slots ~70% busy, DRAM ~25%), so the
     # roofline is the int32 issue peak; the HBM fraction is reported too.
     peaks = {}
     pk = os.path.join(ROOT, "MEASURED_PEAKS.json")

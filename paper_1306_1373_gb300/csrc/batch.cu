@@ -163,8 +163,9 @@ __global__ void __launch_bounds__(256, DCTGB_MINB) k_batch(const __grid_constant
 // The two-lane modes (kernels_pair.cuh): the same per-item descriptor/table
 // slot as k_batch, tiles claimed CHUNK at a time from args.next_tile (or the
 // same contiguous ranges as k_batch when it is null); the samples are read
-// straight from global memory (the 32 resident warps per SM hide the latency
-// that the one-lane kernel hides with cp.async prefetch).  Claimed tiles only
+// straight from global memory (the 24 resident warps per SM hide most of the
+// latency that the one-lane kernel hides with cp.async prefetch: long_scoreboard
+// is 1.5 of the cycles a warp waits per issue).  Claimed tiles only
 // increase, so a warp still meets each item's tiles in order.  CHUNK > 1
 // spares the counter on large batches (many tiles per warp); CHUNK 0 hands out
 // half tiles (units of 16 blocks) where there are fewer tiles than warps.

@@ -8,11 +8,11 @@
 // conflicts).  Against the one-lane tile (kernels.cuh) this halves the code of
 // a tile and the registers: the fused one-lane kernel is 2700 instructions
 // long and waits for instruction fetches (ncu: 1.5 cycles of "no instruction"
-// per issued one, 0.1 here).  What bounds it is issue (66% of cycles, a packed
-// float instruction holding two), with the integer ALU at 60% and the L1 data
-// path at 56%.  At most 80 registers (24 warps per SM): 138.4 us on 8192 x
-// 8192 + 4K 4:2:0 against 142.4 us at 64 registers (32 warps, spills).  The
-// samples wait for the SSE in a per-lane shared-memory slot, and the codes
+// per issued one, 0.1 here).  No pipe is full: issue is busy for 71% of the
+// cycles, the integer ALU 60%, the L1 data path 57%, and the rest is latency that
+// the resident warps do not hide.  At most 80 registers (24 warps per SM): 138.4
+// us on 8192 x 8192 + 4K 4:2:0 against 142.4 us at 64 registers (32 warps,
+// spills).  The samples wait for the SSE in a per-lane shared-memory slot, and the codes
 // leave through the transpose buffer, free between the two transposes, so that
 // a store moves 512 contiguous bytes (8 bytes per lane straight from registers
 // touched 16 cache lines per store; the forward pass alone took 83.1 us that
@@ -43,7 +43,8 @@ constexpr int kParkBytes = 32 * 32;               // each lane's 32 samples, kep
 
 // The part of a QuantSet that a mode reads: [M, Mf, QW, QWc] fused, [M, Mf]
 // forward, [QWi] for the inverse of own codes, [Q, W] for the inverse of any.
-// Batched warps keep only that part, so that 32 warps' slots fit an SM.
+// Batched warps copy only that part, the two-lane ones keep no room for more (the
+// slots of 24 warps take 163 of an SM's 227 KB).
 __host__ __device__ constexpr int pair_tab_first(unsigned mode) {
     return (mode & kLoadPix) ? (int)offsetof(QuantSet, M)
                              : (mode & kOwnCodes) ? (int)offsetof(QuantSet, QWi) : (int)offsetof(QuantSet, Q);
